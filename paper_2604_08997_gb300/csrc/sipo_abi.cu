@@ -1201,7 +1201,7 @@ struct Solver final : SolverBase {
       if (ev) ck(cudaEventRecord(ev[i], s), "event");
     };
     rec(0);
-    k_scalar_step<false><<<1, kThreads, 0, s>>>(st, part);
+    k_scalar_step<false><<<1, kScalarThreads, 0, s>>>(st, part);
     count(1);
     rec(1);
     if (psf) enqueue_psf_q(q, s);
@@ -1238,7 +1238,7 @@ struct Solver final : SolverBase {
     const Geo<C> g = geo();
     const Bufs<S, C> B = bufs();
     const long long nvv = (long long)(V / ze), nvs = (long long)(SN / ze);
-    k_scalar_step<true><<<1, kThreads, 0, s>>>(st, part);
+    k_scalar_step<true><<<1, kScalarThreads, 0, s>>>(st, part);
     count(1);
     if (psf) enqueue_psf_q(q, s);
     launch_project<S, S, C, kFpPrimalCheck, C>(g, psf ? kq : q, B, (C*)nullptr, act_col, zl, s, nbits, rspan);
@@ -1257,7 +1257,7 @@ struct Solver final : SolverBase {
     launch_project<S, S, C, kFpResid, C>(g, psf ? kq : qp, B, (C*)nullptr, act_col, zl, s, nbits, rspan);
     count(1);
     enqueue_certificate(s);
-    k_scalar_check<<<1, kThreads, 0, s>>>(st, part);
+    k_scalar_check<<<1, 32 * kCheckWarps, 0, s>>>(st, part);
     count(1);
     if (ze > 1) {
       k_blend_sino<S, C, z_group<C>()><<<grid_for(nvs), kThreads, 0, s>>>(B, nvs);

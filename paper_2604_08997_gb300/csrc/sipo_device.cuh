@@ -250,9 +250,12 @@ __device__ __forceinline__ void floor_split(float u, float& fl, int& i) {
   i = __float_as_int(t) - 0x4B400000;
   fl = t - 12582912.0f;
 }
+// Double precision the same way with 1.5*2^52 (exact for |u| < 2^31, the int's
+// range): two FP64 additions instead of a rounding and a conversion.
 __device__ __forceinline__ void floor_split(double u, double& fl, int& i) {
-  fl = floor(u);
-  i = int(fl);
+  const double t = __dadd_rd(u, 6755399441055744.0);
+  i = __double2loint(t);
+  fl = t - 6755399441055744.0;
 }
 
 
@@ -261,10 +264,19 @@ __device__ __forceinline__ void floor_split(double u, double& fl, int& i) {
 // one pass over the warps in fixed order; thread 0 writes the block partials
 // to part[slot * kRedBlocks + blockIdx.x].
 // Slots whose bit is set in MAXMASK are reduced with max instead of sum.
-template <int N, unsigned MAXMASK = 0u>
-__device__ __forceinline__ void block_reduce_store(double (&v)[N], double* part, int slot0) {
+// active (the same for the whole block): false where the block had no tile and
+// every value is still zero; it then stores zeros without the FP64 shuffles,
+// which cost a small problem more than its work (1216 blocks, 2 FP64 lanes per
+// clock and SM).  WARPS = 1: only the first warp holds values.
+template <int N, unsigned MAXMASK = 0u, int WARPS = kWarps>
+__device__ __forceinline__ void block_reduce_store(double (&v)[N], double* part, int slot0, bool active = true) {
   __shared__ double red[kWarps][N > 0 ? N : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (!active) {
+    if (threadIdx.x < N) part[(slot0 + threadIdx.x) * kRedBlocks + blockIdx.x] = 0.0;
+    return;
+  }
+  if (warp < WARPS) {
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     double x = v[i];
@@ -276,15 +288,41 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[N], double* part,
     }
     if (lane == 0) red[warp][i] = x;
   }
+  }
   __syncthreads();
   if (threadIdx.x < N) {
     const bool mx = (MAXMASK >> threadIdx.x) & 1u;
     double s = red[0][threadIdx.x];
 #pragma unroll
-    for (int w = 1; w < kWarps; ++w) s = mx ? fmax(s, red[w][threadIdx.x]) : s + red[w][threadIdx.x];
+    for (int w = 1; w < WARPS; ++w) s = mx ? fmax(s, red[w][threadIdx.x]) : s + red[w][threadIdx.x];
     SIPO_DCHECK(isfinite(s) || (mx && s == CUDART_INF), 3);
     part[(slot0 + threadIdx.x) * kRedBlocks + blockIdx.x] = s;
   }
+}
+
+// Sum (or, mx, maximum of non-negative values) of one slot over all kRedBlocks
+// partials by one warp, valid in lane 0.  The additions pair up like a tree
+// over 256 strided sums halved seven times, whatever the number of slots
+// reduced side by side.
+__device__ __forceinline__ double warp_slot(const double* part, int slot, bool mx) {
+  const int lane = threadIdx.x & 31;
+  const double* p = part + (size_t)slot * kRedBlocks;
+  double v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = 0.0;
+#pragma unroll
+  for (int q = 0; q < (kRedBlocks + 255) / 256; ++q)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int at = q * 256 + i * 32 + lane;
+      const double x = at < kRedBlocks ? p[at] : 0.0;
+      v[i] = mx ? fmax(v[i], x) : v[i] + x;
+    }
+  auto join = [&](double a, double b) { return mx ? fmax(a, b) : a + b; };
+  double s = join(join(join(v[0], v[4]), join(v[2], v[6])), join(join(v[1], v[5]), join(v[3], v[7])));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s = join(s, __shfl_down_sync(0xffffffffu, s, o));
+  return s;
 }
 
 // Maximum of one slot over all kRedBlocks partials (non-negative values).

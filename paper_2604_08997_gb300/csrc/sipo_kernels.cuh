@@ -290,51 +290,75 @@ __global__ void k_setup_sums(const uint8_t* __restrict__ lab, const C* __restric
     }
   }
   (void)kase;
-  block_reduce_store<8>(v, part, 0);
+  block_reduce_store<8>(v, part, 0, blockIdx.x * (long long)blockDim.x < n);
 }
 
 // ---------------------------------------------------------- scalar kernels
 // One block.  Gradient step of the scalars from the dual sums (Eqs. 48-49),
 // extrapolation, Halpern weight; outside check steps also the Halpern blend.
+//
+// Two warps: one sums the band partials and steps u~, the other the gel
+// partials and v~, each with its constants loaded and its quotients formed
+// before the sums arrive.  Latency is all there is here (two sums of 1216
+// partials and a few FP64 operations between two operator launches): as one
+// 256-thread block with a shared-memory tree per sum and both scalars in one
+// thread it took 8.3 us a launch.
+constexpr int kScalarThreads = 64;
+
 template <bool CHECK>
-__global__ void __launch_bounds__(kThreads) k_scalar_step(Scal* st, const double* part) {
-  if (st->done) return;
-  const double Sb = block_sum_slot(part, kSlSBand);
-  const double Sg = block_sum_slot(part, kSlSGel);
-  if (threadIdx.x != 0) return;
-  const double om = st->omega;
-  double up = st->u, vp = st->v;
-  if (st->has_u && st->col_u > 0) {
-    up = st->u - kEta / (om * st->col_u) * (st->c_u - Sb);
-    if (up < 0.0) up = 0.0;
+__global__ void __launch_bounds__(kScalarThreads) k_scalar_step(Scal* st, const double* part) {
+  const bool first = threadIdx.x < 32;
+  const int done = st->done;
+  const double om = st->omega, col = first ? st->col_u : st->col_v, grad = first ? st->c_u : st->c_v;
+  const double x = first ? st->u : st->v, x0 = first ? st->u0 : st->v0;
+  const int has = first ? st->has_u : st->has_v;
+  const long long k_in = st->k_in, k = st->k;
+  if (done) return;
+  const bool moves = has && col > 0;
+  const double step = moves ? kEta / (om * col) : 0.0;
+  const double w = (double(k_in) + 1.0) / (double(k_in) + 2.0);
+  const double sum = warp_slot(part, first ? kSlSBand : kSlSGel, false);
+  __syncthreads();  // both warps have read the state
+  if ((threadIdx.x & 31) != 0) return;
+  double xp = x;
+  if (moves) {
+    xp = x - step * (grad - sum);
+    if (xp < (first ? 0.0 : 1.0)) xp = first ? 0.0 : 1.0;  // (a NaN stays)
   }
-  if (st->has_v && st->col_v > 0) {
-    vp = st->v - kEta / (om * st->col_v) * (st->c_v - Sg);
-    if (vp < 1.0) vp = 1.0;
-  }
-  st->up = up;
-  st->vp = vp;
-  st->ubar = 2.0 * up - st->u;
-  st->vbar = 2.0 * vp - st->v;
-  const double w = (double(st->k_in) + 1.0) / (double(st->k_in) + 2.0);
-  st->w = w;
-  if (!CHECK) {
-    st->u = w * st->ubar + (1.0 - w) * st->u0;
-    st->v = w * st->vbar + (1.0 - w) * st->v0;
-    st->k_in += 1;
-    st->k += 1;
+  const double xbar = 2.0 * xp - x;
+  const double xn = w * xbar + (1.0 - w) * x0;
+  if (first) {
+    st->up = xp;
+    st->ubar = xbar;
+    if (!CHECK) st->u = xn;
+    st->w = w;
+    if (!CHECK) {
+      st->k_in = k_in + 1;
+      st->k = k + 1;
+    }
+  } else {
+    st->vp = xp;
+    st->vbar = xbar;
+    if (!CHECK) st->v = xn;
   }
 }
 
 // One block.  KKT of T(z) (Sec. 6.1), termination, Farkas test, restart
 // decision and primal-weight update, then the scalar Halpern blend.
-__global__ void __launch_bounds__(kThreads) k_scalar_check(Scal* st, const double* part) {
+// One warp per slot sums the partials side by side, then one thread decides
+// (24 block-wide sums one after another took 50 of 61 us).
+constexpr int kCheckWarps = kSlFrG - kSlRp2 + 1;
+
+__global__ void __launch_bounds__(32 * kCheckWarps) k_scalar_check(Scal* st, const double* part) {
   if (st->done) return;
-  double s[kNumSlots];
-  for (int i = kSlRp2; i <= kSlFrG; ++i) {
+  __shared__ double s[kNumSlots];
+  {
+    const int i = kSlRp2 + int(threadIdx.x >> 5);
     const bool mx = i == kSlFkNeg || i == kSlFrNeg || i == kSlFkG || i == kSlFrG;
-    s[i] = mx ? block_max_slot(part, i) : block_sum_slot(part, i);
+    const double x = warp_slot(part, i, mx);
+    if ((threadIdx.x & 31) == 0) s[i] = x;
   }
+  __syncthreads();
   if (threadIdx.x != 0) return;
   const double up = st->up, vp = st->vp, u = st->u, v = st->v, u0 = st->u0, v0 = st->v0;
   double om = st->omega;
@@ -496,7 +520,7 @@ __global__ void __launch_bounds__(kThreads) k_cert_vol(Bufs<S, C> b, long long n
     }
     b.cert_q[i] = qv;
   }
-  block_reduce_store<1>(red, b.part, kSlCertObj);
+  block_reduce_store<1>(red, b.part, kSlCertObj, blockIdx.x * (long long)blockDim.x < n);
 }
 
 // One block: the decision from the partials of k_cert_vol and of the
@@ -717,7 +741,7 @@ __global__ void __launch_bounds__(kThreads) k_blend_vol(Bufs<S, C> b, long long 
     store_z<C, C, ZL>(b.d + base, nd);
     store_z<S, C, ZL>(b.q + base, nq);
   }
-  block_reduce_store<2>(red, b.part, kSlSBand);
+  block_reduce_store<2>(red, b.part, kSlSBand, blockIdx.x * (long long)blockDim.x < nvec);
 }
 
 // Stand-alone dual update from a stored d_bar: used when the PSF sits between
@@ -737,7 +761,8 @@ __global__ void __launch_bounds__(kThreads) k_dual(Bufs<S, C> b, const C* __rest
     load_z<C, C, ZL>(dbar + base, db);
     dual_update<S, C, ZL, CHECK>(b, sc, base, db, red);
   }
-  block_reduce_store<NR, CHECK ? kCheckMaxMask : 0u>(red, b.part, CHECK ? kSlRp2 : kSlSBand);
+  block_reduce_store<NR, CHECK ? kCheckMaxMask : 0u>(red, b.part, CHECK ? kSlRp2 : kSlSBand,
+                                                     blockIdx.x * (long long)blockDim.x < nvec);
 }
 
 // --------------------------------------------------------- post-solve
@@ -771,6 +796,11 @@ k_metrics(const C* __restrict__ d, const uint8_t* __restrict__ lab, const float*
   }
   __shared__ double sh[kThreads];
   double vals[8] = {mn_r, mx_r, mx_b, mn_d, sdf, sdd, mn_s, mx_s};
+  if (blockIdx.x * (long long)blockDim.x >= n) {  // no element: the neutral values
+    if (threadIdx.x == 0)
+      for (int q = 0; q < 8; ++q) part[q * kRedBlocks + blockIdx.x] = vals[q];
+    return;
+  }
   for (int q = 0; q < 8; ++q) {
     sh[threadIdx.x] = vals[q];
     __syncthreads();
@@ -795,7 +825,7 @@ __global__ void __launch_bounds__(kThreads) k_dot(const C* __restrict__ a, const
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     v[0] += double(a[i]) * double(b[i]);
-  block_reduce_store<1>(v, part, 0);
+  block_reduce_store<1>(v, part, 0, blockIdx.x * (long long)blockDim.x < n);
 }
 
 }  // namespace sipo
