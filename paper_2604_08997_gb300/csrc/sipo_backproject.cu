@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "sipo_bp_tma.cuh"
+#include "sipo_flat.cuh"
 #include "sipo_launch.h"
 #include "sipo_ops.cuh"
 
@@ -141,6 +142,10 @@ template <typename SI, typename S, typename C, int MODE, typename O>
 void launch_backproject(const Geo<C>& g, const SI* sino, const Bufs<S, C>& b, O* out,
                         const uint8_t* need, int zl, cudaStream_t stream, int tile) {
   constexpr int G = z_group<C>();
+  if (zl == 1 && g.nz <= kFlatMaxZ) {
+    k_backproject_flat<SI, S, C, MODE, O><<<kRedBlocks, kThreads, 0, stream>>>(g, sino, b, out, need);
+    return;
+  }
   if (zl == 2 * G)
     launch_bp_zl<SI, S, C, 2 * G, MODE, O>(g, sino, b, out, need, stream, tile);
   else if (zl == G)

@@ -235,6 +235,62 @@ __device__ __forceinline__ void fp_walk(const Geo<C>& g, const SI* vz, const Nee
   }
 }
 
+// FP64 sums that a projector mode keeps per thread.
+__host__ __device__ constexpr int fp_reductions(int mode) {
+  return mode == kFpPrimalCheck ? 2 : (mode == kFpResid ? 4 : (mode == kFpCert ? 1 : 0));
+}
+
+// What a projector mode does with a finished z-vector of rays (g = acc) at
+// element `base` (z index z0).
+template <typename S, typename C, int ZL, int MODE, typename O>
+__device__ __forceinline__ void fp_finish(const Bufs<S, C>& b, const StepScalars<C>& sc, O* out, size_t base, int z0,
+                                          const C (&acc)[ZL], double* red, unsigned long long* kz_block) {
+  if constexpr (MODE == kFpStore) {
+    store_z<O, C, ZL>(out + base, acc);
+  } else if constexpr (MODE == kFpPrimal) {
+    primal_update<S, C, ZL, false>(b, sc, base, acc, red);
+  } else if constexpr (MODE == kFpPrimalCheck) {
+    primal_update<S, C, ZL, true>(b, sc, base, acc, red);
+  } else if constexpr (MODE == kFpResid) {
+    resid_update<S, C, ZL>(b, base, acc, red);
+  } else if constexpr (MODE == kFpCert) {
+    cert_update<S, C, ZL>(b, base, acc, red);
+  } else {
+    cert_update_z<S, C, ZL>(b, base, z0, acc, kz_block);
+  }
+}
+
+// End of a projector launch: the block's sums (and per-z maxima) to global
+// memory.  active: the block had a tile; WARPS: the warps that hold sums.
+template <int MODE, int WARPS, typename C, typename S, int NR>
+__device__ __forceinline__ void fp_reduce(const Geo<C>& g, const Bufs<S, C>& b, double (&red)[NR],
+                                          unsigned long long* kz_block, bool active) {
+  if constexpr (MODE == kFpCertZ) {
+    __syncthreads();
+    for (int z = threadIdx.x; z < g.nz; z += blockDim.x)
+      if (kz_block[z] != 0ull) atomicMax(b.cert_kz + z, kz_block[z]);
+  }
+  if constexpr (MODE == kFpPrimalCheck) block_reduce_store<2, 0u, WARPS>(red, b.part, kSlFpX, active);
+  if constexpr (MODE == kFpResid) block_reduce_store<4, kResidMaxMask, WARPS>(red, b.part, kSlRd2, active);
+  if constexpr (MODE == kFpCert) block_reduce_store<1, 1u, WARPS>(red, b.part, kSlCertK, active);
+}
+
+// Clips the walked-axis extent [lo, hi] of the ray with offset sj = j - off to
+// its chord through the vial (+1 margin).
+template <typename C>
+__device__ __forceinline__ void fp_ray_span(const Geo<C>& g, C sj, C c, C s, bool rows, int& lo, int& hi) {
+  if (g.r2i < 0) return;
+  C a = fabs(sj) - C(1.5);
+  a = a > C(0) ? a : C(0);
+  const C R = C(g.vial_r);
+  C H = R * R - a * a;
+  H = (H > C(0) ? sqrt(H) : C(0)) + C(1.5);
+  const C mid = rows ? sj * s + g.cy : sj * c + g.cx;
+  const C half = (rows ? fabs(c) : fabs(s)) * H + C(1);
+  lo = max(lo, -ceil_int(-(mid - half)));
+  hi = min(hi, ceil_int(mid + half));
+}
+
 // SI: element type read from `vol`; O: element type written by kFpStore.
 // act_col: per (angle, bin) flag of rays with an active z (solver modes skip
 // the others); nb: packed per-column flags of voxels whose input can be
@@ -252,7 +308,7 @@ k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __r
   const bool use_bits = nb.rows != nullptr;
   if (MODE != kFpStore && b.st->done) return;
   constexpr int ZC = 32 * ZL;
-  constexpr int NR = MODE == kFpPrimalCheck ? 2 : (MODE == kFpResid ? 4 : (MODE == kFpCert ? 1 : 0));
+  constexpr int NR = fp_reductions(MODE);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nzc = (g.nz + ZC - 1) / ZC;
   const int njb = (g.nd + kWarps - 1) / kWarps;
@@ -288,25 +344,10 @@ k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __r
     if (esj != C(0)) {
       const C c = g.cs[2 * k], s = g.cs[2 * k + 1];
       const C jf = C(j);
-      const C sj = jf - g.off;
-      C H = C(0);
-      if (g.r2i >= 0) {
-        C a = fabs(sj) - C(1.5);
-        a = a > C(0) ? a : C(0);
-        const C R = C(g.vial_r);
-        H = R * R - a * a;
-        H = (H > C(0) ? sqrt(H) : C(0)) + C(1.5);
-      }
       const SI* vz = vol + (z0 < g.nz ? z0 : 0);
       const bool rows = fabs(c) >= fabs(s);
       int lo = 0, hi = (rows ? g.ny : g.nx) - 1;
-      if (g.r2i >= 0) {
-        // walked-axis extent of the ray's chord through the vial (+1 margin)
-        const C mid = rows ? sj * s + g.cy : sj * c + g.cx;
-        const C half = (rows ? fabs(c) : fabs(s)) * H + C(1);
-        lo = max(0, -ceil_int(-(mid - half)));
-        hi = min(hi, ceil_int(mid + half));
-      }
+      fp_ray_span<C>(g, jf - g.off, c, s, rows, lo, hi);
       if (rspan) {
         const int2 r = rspan[(size_t)k * g.nd + j];
         lo = max(lo, r.x);
@@ -326,28 +367,9 @@ k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __r
     if (z0 >= g.nz) continue;
     const size_t base = ((size_t)k * g.nd + j) * g.nz + z0;
     SIPO_DCHECK((z0 + z_offset<C, ZL>(ZL - 1) < g.nz), 0);
-    if constexpr (MODE == kFpStore) {
-      store_z<O, C, ZL>(out + base, acc);
-    } else if constexpr (MODE == kFpPrimal) {
-      primal_update<S, C, ZL, false>(b, sc, base, acc, red);
-    } else if constexpr (MODE == kFpPrimalCheck) {
-      primal_update<S, C, ZL, true>(b, sc, base, acc, red);
-    } else if constexpr (MODE == kFpResid) {
-      resid_update<S, C, ZL>(b, base, acc, red);
-    } else if constexpr (MODE == kFpCert) {
-      cert_update<S, C, ZL>(b, base, acc, red);
-    } else {
-      cert_update_z<S, C, ZL>(b, base, z0, acc, kz_block);
-    }
+    fp_finish<S, C, ZL, MODE, O>(b, sc, out, base, z0, acc, red, kz_block);
   }
-  if constexpr (MODE == kFpCertZ) {
-    __syncthreads();
-    for (int z = threadIdx.x; z < g.nz; z += blockDim.x)
-      if (kz_block[z] != 0ull) atomicMax(b.cert_kz + z, kz_block[z]);
-  }
-  if constexpr (MODE == kFpPrimalCheck) block_reduce_store<2>(red, b.part, kSlFpX);
-  if constexpr (MODE == kFpResid) block_reduce_store<4, kResidMaxMask>(red, b.part, kSlRd2);
-  if constexpr (MODE == kFpCert) block_reduce_store<1, 1u>(red, b.part, kSlCertK);
+  fp_reduce<MODE, kWarps>(g, b, red, kz_block, blockIdx.x < ntiles);
 }
 
 // ----------------------------------------------------------- backprojector
@@ -559,7 +581,7 @@ k_backproject(const Geo<C> g, const SI* __restrict__ sino, const Bufs<S, C> b, O
     }
     __syncwarp();
   }
-  if constexpr (MODE == kBpDual) block_reduce_store<2>(red, b.part, kSlSBand);
+  if constexpr (MODE == kBpDual) block_reduce_store<2>(red, b.part, kSlSBand, blockIdx.x < ntiles);
 }
 
 // ------------------------------------------ backprojector with row patterns
@@ -814,7 +836,7 @@ k_backproject2(const Geo<float> g, const SI* __restrict__ sino, const Bufs<S, fl
     }
     __syncwarp();
   }
-  if constexpr (MODE == kBpDual) block_reduce_store<2>(red, b.part, kSlSBand);
+  if constexpr (MODE == kBpDual) block_reduce_store<2>(red, b.part, kSlSBand, blockIdx.x < ntiles);
 }
 
 // ----------------------------------------------------------- ray row spans

@@ -1,6 +1,7 @@
 // Instantiations of the projector P_mu (gather form) for every storage type
 // and epilogue used by the library.
 #include "sipo_launch.h"
+#include "sipo_flat.cuh"
 #include "sipo_ops.cuh"
 
 #include <algorithm>
@@ -50,6 +51,10 @@ void launch_project(const Geo<C>& g, const SI* vol, const Bufs<S, C>& b, O* out,
   constexpr int G = z_group<C>();
   // the slice-mode certificate keeps one 8-byte maximum per z in shared memory
   const size_t dyn = MODE == kFpCertZ ? size_t(g.nz) * sizeof(unsigned long long) : 0;
+  if (zl == 1 && g.nz <= kFlatMaxZ) {
+    k_project_flat<SI, S, C, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, rspan);
+    return;
+  }
   if (zl == 2 * G)
     k_project<SI, S, C, 2 * G, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan);
   else if (zl == G)
