@@ -298,21 +298,26 @@ __device__ __forceinline__ void fp_ray_span(const Geo<C>& g, C sj, C c, C s, boo
 // rows == nullptr to gather every in-vial voxel; rspan: per-ray walked span
 // meeting such columns (nullptr: the whole ray).
 //
-// Tiles (angle, 8 consecutive bins, z segment) are numbered with the angle
-// fastest, so the grid-stride loop gives every block a mix of central bins
-// (long rays) and outer bins (short rays) and the blocks finish together.
+// Tiles (aw consecutive views x 8 / aw consecutive bins, z segment) are
+// numbered with the view fastest, so the grid-stride loop gives every block a
+// mix of central bins (long rays) and outer bins (short rays) and the blocks
+// finish together.  Bound: L1 and L2 delivery, one 16-byte load a lane per tap
+// and z group.  Rays of neighbouring views at one bin run almost on top of
+// each other, so a tile of 4 views x 2 bins meets more of its columns in L1
+// than 8 bins of one view (see launch_project for the measurements).
 template <typename SI, typename S, typename C, int ZL, int MODE, typename O>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, sizeof(C) == 8 ? 2 : 4)
 k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __restrict__ out,
-          const uint8_t* __restrict__ act_col, const NeedBits nb, const int2* __restrict__ rspan) {
+          const uint8_t* __restrict__ act_col, const NeedBits nb, const int2* __restrict__ rspan, int aw) {
   const bool use_bits = nb.rows != nullptr;
   if (MODE != kFpStore && b.st->done) return;
   constexpr int ZC = 32 * ZL;
   constexpr int NR = fp_reductions(MODE);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nzc = (g.nz + ZC - 1) / ZC;
-  const int njb = (g.nd + kWarps - 1) / kWarps;
-  const long long ntiles = (long long)g.na * njb * nzc;
+  const int bw = kWarps / aw;
+  const int njb = (g.nd + bw - 1) / bw, nka = (g.na + aw - 1) / aw;
+  const long long ntiles = (long long)nka * njb * nzc;
   double red[NR > 0 ? NR : 1] = {};
   StepScalars<C> sc{};
   if (MODE == kFpPrimal || MODE == kFpPrimalCheck) sc = read_scalars<C>(b.st);
@@ -326,13 +331,14 @@ k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __r
   }
 
   for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int k = int(t % g.na);
-    const long long t1 = t / g.na;
+    const int k = int(t % nka) * aw + warp % aw;
+    const long long t1 = t / nka;
     const int tz = int(t1 % nzc);
     const int jb = int(t1 / nzc);
-    const int j = jb * kWarps + warp;
+    const int j = jb * bw + warp / aw;
     const int z0 = tz * ZC + lane * ZLayout<C, ZL>::G;
-    if (j >= g.nd) continue;
+    if (aw > 1) __syncthreads();  // keeps the rays of a tile abreast, so that they meet in L1
+    if (j >= g.nd || k >= g.na) continue;
     if (MODE != kFpStore && act_col != nullptr && !act_col[(size_t)k * g.nd + j]) continue;
     const C esj = g.es ? g.es[(size_t)k * g.nd + j] : C(1);
     C acc[ZL];
