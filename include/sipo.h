@@ -244,11 +244,8 @@ int sipo_response_metrics(sipo_ctx *ctx, const sipo_response *M, const float *m_
  * res->cert_slice names the slice.  y_out (nullable) receives y*, the normalised
  * projection of Eq. 18, as [n_angles][n_det][nz] in FP32 (FP64 when storage
  * is SIPO_F64), host or device per y_location.  Blocks until done.  Errors:
- * INVALID_ARG, CUDA, TIMEOUT (a bounded device-side wait of the staged
- * backprojector gave up), NUMERIC (a check found NaN or infinite residuals,
- * e.g. from an infinite imported start; or the staged backprojector's rows did
- * not fit its box, which the geometry cannot produce); the context stays
- * usable. */
+ * INVALID_ARG, CUDA, NUMERIC (a check found NaN or infinite residuals, e.g.
+ * from an infinite imported start); the context stays usable. */
 int sipo_solve(sipo_ctx *ctx, void *y_out, int y_location, sipo_result *res);
 
 /* Warm start, for precision escalation (a reading of the mixed-precision
@@ -428,37 +425,33 @@ int sipo_profile(sipo_ctx *ctx, int iters, double *phase_ms, int n_phases);
 int sipo_phase_count(void);
 const char *sipo_phase_name(int i);
 
-/* Number of entries in the backprojector tile table (for sipo_tolerances.tile_cfg):
- * 0 = 8 voxel columns per warp at 2 blocks/SM, 1 = 4 columns at 2 blocks/SM,
- * 2 = 4 columns at 3 blocks/SM, 3 and 4 = the single-precision row-pattern
- * kernel (4 columns, the rows of each angle in registers, packed FP32
- * multiply-adds) at 2 and 3 blocks/SM, 5 and 6 = the row-pattern kernel fed
- * by tensor-memory (TMA) copies of each angle's detector rows into shared
- * memory, at 3 and 2 blocks/SM, when nz is a multiple of 256 (else entry 4).
- * FP64 contexts run entry 2 for 3-6.  Every entry gives the same sums bit for
- * bit within one precision. */
+/* Number of entries in the backprojector tile table (for sipo_tolerances.tile_cfg).
+ * Single precision: the row-pattern kernel (4 voxel columns a warp, the rows of
+ * each angle in registers, packed FP32 multiply-adds) at 2 blocks/SM (entries 0,
+ * 1, 3) or 3 (2, 4, 5, 6).  FP64: 0 = 8 voxel columns per warp at 2 blocks/SM, 1 =
+ * 4 columns at 2 blocks/SM, 2-6 = 4 columns at 3 blocks/SM.  Volumes of few z
+ * values have one kernel for every entry.  Every entry gives the same sums bit
+ * for bit within one precision. */
 int sipo_tile_count(void);
 
 /* Checked builds (compiled with -DSIPO_CHECKED, the library
  * libsipo_checked.so): synchronises the device and returns the bits of the
  * index and finiteness checks the kernels recorded since the last call (bit 0
- * projector tap column or z offset, bit 1 backprojector detector or staged
+ * projector tap column or z offset, bit 1 backprojector detector
  * row, bit 2 epilogue z offset, bit 3 non-finite FP64 block sum), with bit 30
  * set to mark a checked build, and clears them.  A plain build returns 0.
  * The checks never trap: a violation is recorded and the kernel goes on. */
 unsigned int sipo_check_flags(void);
 
-/* Self-test of the bounded waits of the staged backprojector (table entries 5
- * and 6): one block of `threads` threads (1..1024) on the current device waits
- * on an mbarrier's first phase with a budget of `budget_cycles` SM clock cycles
- * (> 0).  With `arrive` != 0 thread 0 makes the one arrival the barrier expects
- * and every wait ends at once; with `arrive` == 0 nothing completes the phase
- * and every wait gives up after its budget, as a wait on a tensor-memory copy
- * that never lands does in the kernel (where it sets the fault that makes the
- * solve return SIPO_ERR_TIMEOUT).  *timed_out receives the number of threads
- * whose wait gave up.  Returns SIPO_ERR_TIMEOUT when every wait gave up,
- * SIPO_OK when none did, SIPO_ERR_CUDA on a CUDA error, SIPO_ERR_INVALID_ARG
- * for bad arguments.  Synchronises the device; no solver state is touched. */
+/* Self-test of the library's bounded device-side wait: one block of `threads`
+ * threads (1..1024) on the current device waits on an mbarrier's first phase
+ * with a budget of `budget_cycles` SM clock cycles (> 0).  With `arrive` != 0
+ * thread 0 makes the one arrival the barrier expects and every wait ends at
+ * once; with `arrive` == 0 nothing completes the phase and every wait gives up
+ * after its budget.  *timed_out receives the number of threads whose wait gave
+ * up.  Returns SIPO_ERR_TIMEOUT when every wait gave up, SIPO_OK when none did,
+ * SIPO_ERR_CUDA on a CUDA error, SIPO_ERR_INVALID_ARG for bad arguments.
+ * Synchronises the device; no solver state is touched. */
 int sipo_wait_selftest(long long budget_cycles, int arrive, int threads, unsigned int *timed_out);
 
 /* Total kernels this library has launched in this process (graph nodes count

@@ -520,7 +520,7 @@ def sipo_tile_count() -> int:
 
 
 def sipo_wait_selftest(budget_cycles: int, arrive: bool, threads: int = 128) -> tuple[int, int]:
-    """Runs the staged backprojector's bounded mbarrier wait on its own (see
+    """Runs the bounded mbarrier wait on its own (see
     include/sipo.h); returns (library return code, threads whose wait gave
     up).  SIPO_ERR_TIMEOUT is the expected code when `arrive` is False."""
     out = ctypes.c_uint(0)

@@ -157,8 +157,10 @@ struct Solver final : SolverBase {
   sipo_tolerances tol;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  int zl = 1;  // z values per lane of the operator kernels (z_lanes)
-  int ze = 1;  // z values per thread of the element-wise kernels (G or 1)
+  int ze = 1;  // elements per thread of the element-wise kernels
+  // block tiles of the single-precision backprojector: those with a needed
+  // column (solver steps), and all (the plain operator)
+  BpTiles bpt{nullptr, 0, 0}, bpt_all{nullptr, 0, 0};
   int P = 64;
   bool psf = false;
   int bp_nv = 0;     // backprojector tile table entry
@@ -238,8 +240,8 @@ struct Solver final : SolverBase {
     cp = *c;
     tol = *t;
     P = tol.check_every > 0 ? tol.check_every : 64;
-    zl = z_lanes<C>(nz);
-    ze = zl > 1 ? z_group<C>() : 1;
+    // the element-wise kernels run over whole arrays, whatever nz is
+    ze = (V % z_group<C>() == 0 && SN % z_group<C>() == 0) ? z_group<C>() : 1;
     if (s) {
       stream = s;
     } else {
@@ -435,7 +437,6 @@ struct Solver final : SolverBase {
     ck(cudaGetLastError(), "Farkas test");
     ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
     ck(cudaStreamSynchronize(stream), "Farkas test");
-    check_bp_fault();
     const int cert = h_st->cert;
     if (slice) *slice = cert ? h_st->cert_z : -1;
     init_state();
@@ -453,7 +454,7 @@ struct Solver final : SolverBase {
     k_import_primal<S, C><<<grid_for((long long)SN), kThreads, 0, stream>>>(ts, col, yp, C(scale), (long long)SN);
     ck(cudaFreeAsync(ts, stream), "free");
     // d = A^T y with the operator of a check step's plain backprojection
-    launch_backproject<S, S, C, kBpStore, C>(g, yp, B, psf ? braw : dp, need, zl, stream, bp_nv);
+    launch_backproject<S, S, C, kBpStore, C>(g, yp, B, psf ? braw : dp, need, stream, bpt, bp_nv);
     if (psf) psf3<C, C>(braw, dp, t1, t2, -1, stream);
     count(2);
     if (up_in || lo_in) {
@@ -853,6 +854,51 @@ struct Solver final : SolverBase {
     }
   }
 
+  // ------------------------------------------------- backprojector tiles
+  // Tiles of k_backproject2 with a column in `cols` ([y][x] flags, host), for
+  // 8 >> split rows a tile.
+  std::vector<int> bp_tile_list(const std::vector<uint8_t>& cols, int split) const {
+    const int nrow = kWarps >> split, ntx = (nx + kBp2NV - 1) / kBp2NV, nty = (ny + nrow - 1) / nrow;
+    std::vector<int> list;
+    for (int ty = 0; ty < nty; ++ty)
+      for (int tx = 0; tx < ntx; ++tx) {
+        bool any = false;
+        for (int y = ty * nrow; y < std::min(ny, (ty + 1) * nrow) && !any; ++y)
+          for (int x = tx * kBp2NV; x < std::min(nx, (tx + 1) * kBp2NV) && !any; ++x) any = cols[size_t(y) * nx + x];
+        if (any) list.push_back(ty * ntx + tx);
+      }
+    return list;
+  }
+
+  // Chooses the view split (by shape and target alone, so that sums do not
+  // depend on timing) and lists the solver's tiles.
+  void choose_bp_tiles() {
+    if constexpr (sizeof(C) == 8) return;
+    int T = 1;
+    with_z_form<C>(nz, z_group_for<C>(nz, (const C*)nullptr, (const C*)nullptr), [&](auto f) { T = decltype(f)::T; });
+    const long long nzc = (nz + T - 1) / T;
+    std::vector<uint8_t> cols(size_t(nx) * ny);
+    ck(cudaMemcpyAsync(cols.data(), need, cols.size(), cudaMemcpyDeviceToHost, stream), "need");
+    ck(cudaStreamSynchronize(stream), "need");
+    const long long want = (long long)(1.75 * device_sms() * 3);
+    std::vector<int> list;
+    for (bpt.split = 0;; ++bpt.split) {
+      list = bp_tile_list(cols, bpt.split);
+      if ((long long)list.size() * nzc >= want || bpt.split == 3) break;
+    }
+    int* d = dalloc<int>(list.size());
+    ck(cudaMemcpyAsync(d, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, stream), "tiles");
+    ck(cudaStreamSynchronize(stream), "tiles");
+    bpt.list = d;
+    bpt.n = int(list.size());
+    const double share = vial_r > 0 ? std::min(1.0, 3.14159265 * vial_r * vial_r / (double(nx) * ny)) : 1.0;
+    for (bpt_all.split = 0; bpt_all.split < 3; ++bpt_all.split) {
+      const int nrow = kWarps >> bpt_all.split;
+      const double tiles = share * ((nx + kBp2NV - 1) / kBp2NV) * ((ny + nrow - 1) / nrow) * double(nzc);
+      if (tiles >= double(want)) break;
+    }
+  }
+
   // -------------------------------------------------------------- setup
   void setup(const float* fT_src, const float* fL_src, const float* fU_src) override {
     if (psf) {
@@ -988,6 +1034,7 @@ struct Solver final : SolverBase {
         k_need_cols<<<gc, kThreads, 0, stream>>>(lab, need, nx, ny, nz);
       }
     }
+    choose_bp_tiles();
     rspan = dalloc<int2>(size_t(na) * nd);
     launch_ray_spans<C>(geo(), need, rspan, stream);
     {
@@ -999,6 +1046,7 @@ struct Solver final : SolverBase {
       nbits.cols = bc;
       nbits.wr = wr;
       nbits.wc = wc;
+      nbits.spread = psf;
     }
     // iterate storage
     y = dalloc<S>(SN); y0 = dalloc<S>(SN); yp = dalloc<S>(SN); ybar = dalloc<S>(SN);
@@ -1028,7 +1076,7 @@ struct Solver final : SolverBase {
       k_convert<float, C><<<gv, kThreads, 0, stream>>>(fT, t1, (long long)V);
       src = t1;
     }
-    launch_project<C, C, C, kFpStore, C>(g, src, Bufs<C, C>{}, gp, nullptr, zl, stream);
+    launch_project<C, C, C, kFpStore, C>(g, src, Bufs<C, C>{}, gp, nullptr, stream);
     const int gs = grid_for((long long)SN);
     k_mask<C><<<gs, kThreads, 0, stream>>>(gp, mask, g0, (long long)SN);
     k_act_cols<<<grid_for((long long)na * nd), kThreads, 0, stream>>>(mask, act_col, (long long)na * nd, nz);
@@ -1037,17 +1085,17 @@ struct Solver final : SolverBase {
     if (psf) {
       psf3<C, C>(t1, t2, t3, braw, -1, stream);
       ck(cudaMemsetAsync(braw, 0, V * sizeof(C), stream), "memset");
-      launch_project<C, C, C, kFpStore, C>(g, t2, Bufs<C, C>{}, col, nullptr, zl, stream);
+      launch_project<C, C, C, kFpStore, C>(g, t2, Bufs<C, C>{}, col, nullptr, stream);
     } else {
-      launch_project<C, C, C, kFpStore, C>(g, t1, Bufs<C, C>{}, col, nullptr, zl, stream);
+      launch_project<C, C, C, kFpStore, C>(g, t1, Bufs<C, C>{}, col, nullptr, stream);
     }
     k_apply_mask<C><<<gs, kThreads, 0, stream>>>(col, mask, (long long)SN);
     // row abs-sums of A^T over active rays: A^T 1_act = K P^T 1_act
     if (psf) {
-      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, t1, nullptr, zl, stream);
+      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, t1, nullptr, stream, bpt_all);
       psf3<C, C>(t1, row, t2, t3, -1, stream);
     } else {
-      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, row, nullptr, zl, stream);
+      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, row, nullptr, stream, bpt_all);
     }
     (void)B;
     // setup sums
@@ -1085,9 +1133,9 @@ struct Solver final : SolverBase {
       if (psf) {
         psf3<C, C>(t1, t2, t3, braw, -1, stream);
         ck(cudaMemsetAsync(braw, 0, V * sizeof(C), stream), "memset");
-        launch_project<C, C, C, kFpStore, C>(g, t2, Bufs<C, C>{}, cert_b, nullptr, zl, stream);
+        launch_project<C, C, C, kFpStore, C>(g, t2, Bufs<C, C>{}, cert_b, nullptr, stream);
       } else {
-        launch_project<C, C, C, kFpStore, C>(g, t1, Bufs<C, C>{}, cert_b, nullptr, zl, stream);
+        launch_project<C, C, C, kFpStore, C>(g, t1, Bufs<C, C>{}, cert_b, nullptr, stream);
       }
       cert_B = cp.kase == SIPO_CASE2 ? double(n_band) * band_rhs : (fu ? sums[7] : up_ratio * sums[2]);
       count(3);
@@ -1159,6 +1207,7 @@ struct Solver final : SolverBase {
       bp_nv = tol.tile_cfg;
       return;
     }
+    if (bp_flat<C>(nz)) return;  // no tiles to choose from
     const TileKey key{nx, ny, nz, na, nd, tol.storage, psf ? 1 : 0};
     {
       std::lock_guard<std::mutex> lock(g_tile_mutex);
@@ -1173,6 +1222,8 @@ struct Solver final : SolverBase {
     cudaEvent_t ev[7];
     for (auto& e : ev) ck(cudaEventCreate(&e), "event");
     for (int tile = 0; tile < kBpTiles; ++tile) {
+      // entries that run the same kernel as another one
+      if (sizeof(C) == 8 ? tile > 2 : (tile != 3 && tile != 4)) continue;
       bp_nv = tile;
       init_state();
       float tot = 0.0f;
@@ -1206,18 +1257,18 @@ struct Solver final : SolverBase {
     rec(1);
     if (psf) enqueue_psf_q(q, s);
     rec(2);
-    launch_project<S, S, C, kFpPrimal, C>(g, psf ? kq : q, B, (C*)nullptr, act_col, zl, s, nbits, rspan);
+    launch_project<S, S, C, kFpPrimal, C>(g, psf ? kq : q, B, (C*)nullptr, act_col, s, nbits, rspan);
     count(1);
     rec(3);
     if (psf) {
-      launch_backproject<S, S, C, kBpStore, C>(g, ybar, B, braw, need, zl, s, bp_nv);
+      launch_backproject<S, S, C, kBpStore, C>(g, ybar, B, braw, need, s, bpt, bp_nv);
       count(1);
       rec(4);
       psf3<C, C>(braw, t3, t1, t2, -1, s);
       rec(5);
       dual_launch<false>(B, t3, nvv, s);
     } else {
-      launch_backproject<S, S, C, kBpDual, C>(g, ybar, B, (C*)nullptr, need, zl, s, bp_nv);
+      launch_backproject<S, S, C, kBpDual, C>(g, ybar, B, (C*)nullptr, need, s, bpt, bp_nv);
       count(1);
       rec(4);
       rec(5);
@@ -1241,20 +1292,20 @@ struct Solver final : SolverBase {
     k_scalar_step<true><<<1, kScalarThreads, 0, s>>>(st, part);
     count(1);
     if (psf) enqueue_psf_q(q, s);
-    launch_project<S, S, C, kFpPrimalCheck, C>(g, psf ? kq : q, B, (C*)nullptr, act_col, zl, s, nbits, rspan);
+    launch_project<S, S, C, kFpPrimalCheck, C>(g, psf ? kq : q, B, (C*)nullptr, act_col, s, nbits, rspan);
     count(1);
     if (psf) {
-      launch_backproject<S, S, C, kBpStore, C>(g, ybar, B, braw, need, zl, s, bp_nv);
+      launch_backproject<S, S, C, kBpStore, C>(g, ybar, B, braw, need, s, bpt, bp_nv);
       count(1);
       psf3<C, C>(braw, t3, t1, t2, -1, s);
       dual_launch<true>(B, t3, nvv, s);
       enqueue_psf_q(qp, s);
     } else {
-      launch_backproject<S, S, C, kBpStore, C>(g, ybar, B, braw, need, zl, s, bp_nv);
+      launch_backproject<S, S, C, kBpStore, C>(g, ybar, B, braw, need, s, bpt, bp_nv);
       count(1);
       dual_launch<true>(B, braw, nvv, s);
     }
-    launch_project<S, S, C, kFpResid, C>(g, psf ? kq : qp, B, (C*)nullptr, act_col, zl, s, nbits, rspan);
+    launch_project<S, S, C, kFpResid, C>(g, psf ? kq : qp, B, (C*)nullptr, act_col, s, nbits, rspan);
     count(1);
     enqueue_certificate(s);
     k_scalar_check<<<1, 32 * kCheckWarps, 0, s>>>(st, part);
@@ -1281,7 +1332,7 @@ struct Solver final : SolverBase {
         psf3<C, C>(cert_q, t3, t1, t2, -1, s);
         cq = t3;
       }
-      launch_project<C, S, C, kFpCertZ, C>(g, cq, B, (C*)nullptr, act_col, zl, s, nbits, rspan);
+      launch_project<C, S, C, kFpCertZ, C>(g, cq, B, (C*)nullptr, act_col, s, nbits, rspan);
       k_cert_decide_z<<<1, kThreads, 0, s>>>(st, cert_pz, kCertBlocks, nz, cert_kz, cert_Bz);
       count(3);
     } else if (cert_on) {
@@ -1291,7 +1342,7 @@ struct Solver final : SolverBase {
         psf3<C, C>(cert_q, t3, t1, t2, -1, s);
         cq = t3;
       }
-      launch_project<C, S, C, kFpCert, C>(g, cq, B, (C*)nullptr, act_col, zl, s, nbits, rspan);
+      launch_project<C, S, C, kFpCert, C>(g, cq, B, (C*)nullptr, act_col, s, nbits, rspan);
       k_cert_decide<<<1, kThreads, 0, s>>>(st, part);
       count(3);
     }
@@ -1353,7 +1404,6 @@ struct Solver final : SolverBase {
   void finish_solve(void* y_out, int loc, sipo_result* res) override {
     ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
     ck(cudaStreamSynchronize(stream), "solve");
-    check_bp_fault();
     if (!h_st->done) {
       final_check();
       ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
@@ -1366,7 +1416,7 @@ struct Solver final : SolverBase {
     // f~* = A^T y* of the returned point, recomputed by one plain application
     // of the operator: the iterations carry d by linearity (d+ = (d_bar + d) / 2),
     // which drifts from A^T y by rounding over many steps in FP32
-    launch_backproject<S, S, C, kBpStore, C>(geo(), yp, bufs(), psf ? braw : dp, need, zl, stream, bp_nv);
+    launch_backproject<S, S, C, kBpStore, C>(geo(), yp, bufs(), psf ? braw : dp, need, stream, bpt, bp_nv);
     count(1);
     if (psf) psf3<C, C>(braw, dp, t1, t2, -1, stream);
     // metrics of d = A^T y at the returned point (Eqs. 6-8, 27, 46)
@@ -1410,15 +1460,6 @@ struct Solver final : SolverBase {
     res->cert_slice = h.status == 1 ? h.cert_z : -1;
   }
 
-  // A bounded wait inside the staged backprojector gave up (bit 0), or an
-  // angle's rows did not fit its box (bit 1): the sums of that launch are not
-  // valid, so the solve is an error.
-  void check_bp_fault() {
-    const unsigned int f = bp3_fault_take();
-    if (f & 1u) fail(SIPO_ERR_TIMEOUT, "backprojector: a wait on a tensor-memory copy timed out");
-    if (f) fail(SIPO_ERR_NUMERIC, "backprojector: detector rows outside the staged box");
-  }
-
   // copies n elements of S (converted to C) to out (host or device)
   template <typename T>
   void copy_out(const T* src, size_t n, void* out, int loc, C* tmp) {
@@ -1443,7 +1484,7 @@ struct Solver final : SolverBase {
       psf3<C, C>(src, t3, t1, t2, -1, s);
       src = t3;
     }
-    launch_project<C, C, C, kFpStore, C>(g, src, Bufs<C, C>{}, static_cast<C*>(sino), nullptr, zl, s);
+    launch_project<C, C, C, kFpStore, C>(g, src, Bufs<C, C>{}, static_cast<C*>(sino), nullptr, s);
     count(1);
     ck(cudaGetLastError(), "project");
   }
@@ -1452,12 +1493,12 @@ struct Solver final : SolverBase {
     const Geo<C> g = geo();
     if (psf) {
       ensure_temps();
-      launch_backproject<C, C, C, kBpStore, C>(g, static_cast<const C*>(sino), Bufs<C, C>{}, t3, nullptr, zl, s,
+      launch_backproject<C, C, C, kBpStore, C>(g, static_cast<const C*>(sino), Bufs<C, C>{}, t3, nullptr, s, bpt_all,
                                                bp_nv);
       psf3<C, C>(t3, static_cast<C*>(vol), t1, t2, -1, s);
     } else {
       launch_backproject<C, C, C, kBpStore, C>(g, static_cast<const C*>(sino), Bufs<C, C>{},
-                                               static_cast<C*>(vol), nullptr, zl, s, bp_nv);
+                                               static_cast<C*>(vol), nullptr, s, bpt_all, bp_nv);
     }
     count(1);
     ck(cudaGetLastError(), "backproject");
@@ -1480,7 +1521,7 @@ struct Solver final : SolverBase {
     double* pg = dalloc_part();
     // b = P_mu^T sino, recomputed (not stored by the forward pass)
     launch_backproject<C, C, C, kBpStore, C>(geo(), static_cast<const C*>(sino), Bufs<C, C>{}, tvol, nullptr,
-                                             zl, s);
+                                             s, bpt_all, bp_nv);
     count(1);
     for (int a = 0; a < 3; ++a) {
       grad[a] = 0.0;

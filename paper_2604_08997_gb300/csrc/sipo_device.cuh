@@ -127,6 +127,14 @@ __device__ __forceinline__ void load_group(const S* __restrict__ p, C* v) {
         v[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
       }
     }
+  } else if constexpr (kBytes == 8 && sizeof(S) == 4) {
+    const float2 r = __ldg(reinterpret_cast<const float2*>(p));
+    v[0] = r.x;
+    v[1] = r.y;
+  } else if constexpr (kBytes == 4 && sizeof(S) == 2) {
+    const uint32_t r = __ldg(reinterpret_cast<const uint32_t*>(p));
+    v[0] = __uint_as_float(r << 16);
+    v[1] = __uint_as_float(r & 0xffff0000u);
   } else if constexpr (kBytes == 8 && sizeof(S) == 2) {
     const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
     v[0] = __uint_as_float(r.x << 16);
@@ -146,6 +154,11 @@ __device__ __forceinline__ void store_group(S* __restrict__ p, const C* v) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
   } else if constexpr (kBytes == 16 && sizeof(S) == 8) {
     *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+  } else if constexpr (kBytes == 8 && sizeof(S) == 4) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  } else if constexpr (sizeof(S) == 2 && G == 2) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(v[0], v[1]);
+    *reinterpret_cast<__nv_bfloat162*>(p) = h;
   } else if constexpr (sizeof(S) == 2 && (G == 4 || G == 8)) {
     uint32_t w[G / 2];
 #pragma unroll
@@ -196,6 +209,73 @@ __device__ __forceinline__ void load_labels(const uint8_t* __restrict__ p, uint8
       for (int j = 0; j < L::G; ++j) lab[q * L::G + j] = pq[j];
     }
   }
+}
+
+// ------------------------------------------------------- z forms of operators
+// How a warp covers z in the operator kernels: NG groups of G elements a lane,
+// group q of the lanes spanning 32 G consecutive values, T = 32 G NG values a
+// tile.  G is set by alignment (4, 2 or 1 floats as nz and the buffers allow), NG by
+// the extent (z_form in sipo_launch.h).  RAGGED = false: nz is a multiple of T
+// and every group starts at q * 32 G.  RAGGED = true: groups and tiles that
+// would run past the end of the column start earlier, so that every load
+// stays inside it, and the values that a preceding group or tile owns are
+// loaded again but not finished (fresh() is false there).
+template <int G_, int NG_, bool RAGGED_>
+struct ZForm {
+  static constexpr int G = G_, NG = NG_, ZL = G_ * NG_, T = 32 * G_ * NG_;
+  static constexpr bool kRagged = RAGGED_;
+};
+
+template <typename Z>
+struct ZSpan {
+  int z0;              // the lane's first element of group 0
+  int off[Z::NG];      // start of group q from group 0 (the same for all lanes)
+  unsigned fresh;      // bit q: the lane owns its elements of group q
+  __device__ __forceinline__ int at(int q) const { return Z::kRagged ? off[q] : q * 32 * Z::G; }
+  __device__ __forceinline__ bool owns(int q) const { return !Z::kRagged || ((fresh >> q) & 1u); }
+  __device__ __forceinline__ void init(int nz, int tz) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (!Z::kRagged) {
+      z0 = tz * Z::T + lane * Z::G;
+      fresh = ~0u;
+    } else {
+      const int t0 = min(tz * Z::T, max(nz - Z::T, 0));
+      const bool idle = lane * Z::G >= nz;
+      z0 = idle ? 0 : t0 + lane * Z::G;
+      fresh = 0u;
+#pragma unroll
+      for (int q = 0; q < Z::NG; ++q) {
+        off[q] = min(q * 32 * Z::G, max(nz - 32 * Z::G, 0));
+        const int first = off[q] < q * 32 * Z::G ? q * 32 * Z::G : tz * Z::T;
+        if (!idle && z0 + off[q] >= first) fresh |= 1u << q;
+      }
+    }
+  }
+};
+
+// The lane's values; p points at its first element of group 0.
+template <typename Z, typename S, typename C>
+__device__ __forceinline__ void load_zf(const S* __restrict__ p, const ZSpan<Z>& zs, C (&v)[Z::ZL]) {
+#pragma unroll
+  for (int q = 0; q < Z::NG; ++q) load_group<S, C, Z::G>(p + zs.at(q), v + q * Z::G);
+}
+
+// The same for the owned groups only (zeros elsewhere).
+template <typename Z, typename S, typename C>
+__device__ __forceinline__ void load_owned(const S* __restrict__ p, const ZSpan<Z>& zs, C (&v)[Z::ZL]) {
+#pragma unroll
+  for (int q = 0; q < Z::NG; ++q) {
+#pragma unroll
+    for (int i = 0; i < Z::G; ++i) v[q * Z::G + i] = C(0);
+    if (zs.owns(q)) load_group<S, C, Z::G>(p + zs.at(q), v + q * Z::G);
+  }
+}
+
+template <typename Z, typename S, typename C>
+__device__ __forceinline__ void store_owned(S* __restrict__ p, const ZSpan<Z>& zs, const C (&v)[Z::ZL]) {
+#pragma unroll
+  for (int q = 0; q < Z::NG; ++q)
+    if (zs.owns(q)) store_group<S, C, Z::G>(p + zs.at(q), v + q * Z::G);
 }
 
 // ------------------------------------------------------------------ geometry

@@ -23,10 +23,6 @@
 
 namespace sipo {
 
-// z extents that take these kernels when the z-lane kernels would run their
-// one-value-per-lane path (zl == 1).
-constexpr int kFlatMaxZ = 8;
-
 // Lines per chunk of a warp, so that a block's staged columns stay below 48 KB
 // in both compute types.
 template <typename C> constexpr int flat_chunk() { return sizeof(C) == 8 ? 8 : 16; }
@@ -61,14 +57,18 @@ __device__ __forceinline__ bool flat_hit(double w) { return unsigned(__double2hi
 // backprojector's two taps, so that a voxel is read and weighed once for both
 // bins.  ROWS: the ray is walked along y (lines are rows, read from global
 // memory: the lanes' voxels are neighbours along x); otherwise along x, the
-// chunk's columns staged in shared memory with reads along x.  EDGE: the tile
-// with bin -1.  ATT: attenuation.  Z1: one z value (compile-time stride).
-template <bool ROWS, bool EDGE, bool ATT, bool Z1, typename SI, typename C>
+// chunk's columns staged in shared memory with reads along x.  EDGE: any tile
+// (bin -1 among its bins, any z stride, inputs that reach outside the vial);
+// otherwise one z value.  ATT: attenuation.  wide: the input vanishes where it
+// should not count except outside the vial, where each ray counts it on its own
+// lines [mine.x, mine.y] (a solver's blurred duals; as k_project with NeedBits).
+template <bool ROWS, bool EDGE, bool ATT, typename SI, typename C>
 __device__ __forceinline__ void flat_walk(const Geo<C>& g, const SI* vz, int k, C jf, C c, C s, int lo, int hi,
-                                          C (*stage)[flat_chunk<C>() + 1], C& own, C& next) {
+                                          bool wide, int2 mine, C (*stage)[flat_chunk<C>() + 1], C& own, C& next) {
   constexpr int kCh = flat_chunk<C>(), kRows = flat_rows<C>();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nz = Z1 ? 1 : g.nz;
+  const int nz = EDGE ? g.nz : 1;
+  const int2 above = make_int2(__shfl_down_sync(0xffffffffu, mine.x, 1), __shfl_down_sync(0xffffffffu, mine.y, 1));
   const C a = ROWS ? c : s;
   const C inv_a = C(1) / a;
   // first candidate on a line: ceil(base + slope line)
@@ -107,7 +107,8 @@ __device__ __forceinline__ void flat_walk(const Geo<C>& g, const SI* vz, int k, 
       float cf;
       int i0;
       ceil_split(fmaf(lf, slope, base), cf, i0);
-      const int2 sp = ROWS ? g.xspan[line] : g.yspan[line];
+      int2 sp = ROWS ? g.xspan[line] : g.yspan[line];
+      if (EDGE && wide) sp = make_int2(0, (ROWS ? g.nx : g.ny) - 1);
       const unsigned len = unsigned(sp.y - sp.x + 1) & ~unsigned((sp.y - sp.x) >> 31);  // 0: empty span
       const C f0 = flat_coord(cf, i0, ROWS ? g.cx : g.cy);
       C sh;
@@ -148,6 +149,10 @@ __device__ __forceinline__ void flat_walk(const Geo<C>& g, const SI* vz, int k, 
             w *= e;
           }
         }
+        if (EDGE && wide) {
+          if (line < mine.x || line > mine.y) w0 = C(0);
+          if (line < above.x || line > above.y) w = C(0);
+        }
         own = fma(w0, v, own);
         next = fma(w, v, next);
       }
@@ -158,7 +163,7 @@ __device__ __forceinline__ void flat_walk(const Geo<C>& g, const SI* vz, int k, 
 template <typename SI, typename S, typename C, int MODE, typename O>
 __global__ void __launch_bounds__(kThreads, sizeof(C) == 8 ? 4 : 5)
 k_project_flat(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __restrict__ out,
-               const uint8_t* __restrict__ act_col, const int2* __restrict__ rspan) {
+               const uint8_t* __restrict__ act_col, const int2* __restrict__ rspan, bool wide) {
   if (MODE != kFpStore && b.st->done) return;
   constexpr int NR = fp_reductions(MODE);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -198,20 +203,22 @@ k_project_flat(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O
       }
       if (lo > hi) { lo = 0x3fffffff; hi = -1; }
     }
+    const int2 mine = make_int2(lo, hi);
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     const SI* vz = vol + z;
     C own = C(0), next = C(0);
     if (lo <= hi) {
       const bool att = g.ex != nullptr;
-#define SIPO_FLAT(R, E, A, Z) flat_walk<R, E, A, Z, SI, C>(g, vz, k, jf, c, s, lo, hi, stage[warp], own, next)
-      if (jb == 0 || g.nz != 1) {  // the general form: floors compared, runtime z stride
-        if (rows) { if (att) SIPO_FLAT(true, true, true, false); else SIPO_FLAT(true, true, false, false); }
-        else { if (att) SIPO_FLAT(false, true, true, false); else SIPO_FLAT(false, true, false, false); }
+#define SIPO_FLAT(R, E, A) \
+  flat_walk<R, E, A, SI, C>(g, vz, k, jf, c, s, lo, hi, wide, mine, stage[warp], own, next)
+      if (jb == 0 || g.nz != 1 || wide) {
+        if (rows) { if (att) SIPO_FLAT(true, true, true); else SIPO_FLAT(true, true, false); }
+        else { if (att) SIPO_FLAT(false, true, true); else SIPO_FLAT(false, true, false); }
       } else if (rows) {
-        if (att) SIPO_FLAT(true, false, true, true); else SIPO_FLAT(true, false, false, true);
+        if (att) SIPO_FLAT(true, false, true); else SIPO_FLAT(true, false, false);
       } else {
-        if (att) SIPO_FLAT(false, false, true, true); else SIPO_FLAT(false, false, false, true);
+        if (att) SIPO_FLAT(false, false, true); else SIPO_FLAT(false, false, false);
       }
 #undef SIPO_FLAT
     }
@@ -224,7 +231,10 @@ k_project_flat(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O
 #pragma unroll
       for (int w = 1; w < kWarps; ++w) tot[0] += psum[w][lane];
       tot[0] *= esj;
-      fp_finish<S, C, 1, MODE, O>(b, sc, out, ((size_t)k * g.nd + j) * g.nz + z, z, tot, red, kz_block);
+      ZSpan<ZForm<1, 1, false>> zs;
+      zs.z0 = z;
+      fp_finish<S, C, ZForm<1, 1, false>, MODE, O>(b, sc, out, ((size_t)k * g.nd + j) * g.nz + z, zs, tot, red,
+                                                   kz_block);
     }
   }
   fp_reduce<MODE, 1>(g, b, red, kz_block, blockIdx.x < ntiles);

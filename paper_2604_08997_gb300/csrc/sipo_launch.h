@@ -9,14 +9,12 @@
 
 namespace sipo {
 
-// zl: z values per lane (z_lanes<C>(nz) picks it): 2G or G, G = 16 bytes of
-// compute elements, for the vector paths, 1 for the scalar path.
 // nb: packed per-column flags of voxels whose input may be non-zero (rows ==
 // nullptr: every in-vial voxel); rspan: per-ray walked-axis span holding such
 // columns (nullptr: whole ray).
 template <typename SI, typename S, typename C, int MODE, typename O>
 void launch_project(const Geo<C>& g, const SI* vol, const Bufs<S, C>& b, O* out,
-                    const uint8_t* act_col, int zl, cudaStream_t stream,
+                    const uint8_t* act_col, cudaStream_t stream,
                     const NeedBits& nb = NeedBits{}, const int2* rspan = nullptr);
 
 // Packs need[y][x] into the row-major and column-major bit arrays of NeedBits.
@@ -27,19 +25,12 @@ void launch_need_bits(const uint8_t* need, uint32_t* rows, uint32_t* cols, int n
 template <typename C>
 void launch_ray_spans(const Geo<C>& g, const uint8_t* need, int2* out, cudaStream_t stream);
 
-// tile: entry of the backprojector tile table (0: 8 columns per warp, 2
-// blocks/SM; 1: 4 columns, 2 blocks/SM; 2: 4 columns, 3 blocks/SM; 3, 4: the
-// single-precision row-pattern kernel at 2 and 3 blocks/SM, entry 2 in FP64;
-// 5, 6: the row-pattern kernel with rows staged by tensor-memory copies, at 3
-// and 2 blocks/SM, for nz a multiple of 256, else entry 4).
+// tile: entry of the backprojector tile table.  FP64: 0 = 8 columns per warp, 2
+// blocks/SM; 1 = 4 columns, 2 blocks/SM; 2-6 = 4 columns, 3 blocks/SM.  Single
+// precision: the row-pattern kernel at 2 (0, 1, 3) or 3 (2, 4, 5, 6) blocks/SM.
 constexpr int kBpTiles = 7;
 
-// Reads and clears the fault flag of the staged backprojector (nonzero: a
-// bounded wait on a tensor-memory copy gave up; the launch's sums are not
-// valid).  Synchronous: call outside stream capture.
-unsigned int bp3_fault_take();
-
-// Runs the bounded mbarrier wait of the staged backprojector on its own: one
+// Runs the bounded mbarrier wait (sipo_wait.cuh) on its own: one
 // block of `threads` threads waits `budget` cycles on a barrier that receives
 // its one arrival only if `arrive`; *timed_out = threads whose wait gave up.
 // 0 on success, -1 on a CUDA error.  Synchronous.
@@ -51,17 +42,69 @@ unsigned int check_flags_project();
 unsigned int check_flags_backproject();
 template <typename SI, typename S, typename C, int MODE, typename O>
 void launch_backproject(const Geo<C>& g, const SI* sino, const Bufs<S, C>& b, O* out,
-                        const uint8_t* need, int zl, cudaStream_t stream, int tile = 0);
+                        const uint8_t* need, cudaStream_t stream, const BpTiles& tiles, int tile = 0);
+
+// z extents that take the kernels of sipo_flat.cuh (lanes over bins or voxels):
+// below these the z lanes of the other kernels idle more than the flat ones
+// repeat weights.  200 x 200, 300 views, us, z lanes / flat: single precision,
+// projector 274 / 115 at nz = 4, 277 / 246 at 8, 279 / 349 at 12; backprojector
+// 317 / 149 at 8, 317 / 209 at 12, 319 / 411 at 16; double precision, projector
+// 2696 / 1859 at 4, 2696 / 2738 at 6; backprojector 2387 / 1950 at 8, 2480 / 2879 at 12.
+template <typename C> inline bool fp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 5 : 8); }
+template <typename C> inline bool bp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 9 : 12); }
 
 // Group size G of the z layout (elements of C in 16 bytes).
 template <typename C> constexpr int z_group() { return 16 / int(sizeof(C)); }
 
-// z values per lane for a z extent nz: two groups when a warp's 64 G values
-// tile nz exactly, one group when nz is a multiple of G (the last warp of a
-// column may then be partly idle, lane by lane), else the scalar path.
-template <typename C> inline int z_lanes(int nz) {
-  constexpr int G = z_group<C>();
-  return nz % (64 * G) == 0 ? 2 * G : (nz % G == 0 ? G : 1);
+// Largest group of z values (elements of C in at most 16 bytes) that nz and the
+// buffers' alignment allow: every z column then starts on a group boundary.
+template <typename C, typename A, typename B>
+inline int z_group_for(int nz, const A* a, const B* b) {
+  int G = z_group<C>();
+  const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+  while (G > 1 && (nz % G != 0 || pa % (G * sizeof(A)) != 0 || pb % (G * sizeof(B)) != 0)) G /= 2;
+  return G;
+}
+
+// Calls f(ZForm) with the z form for extent nz and groups of at most gmax values
+// (see ZForm): the form with the least tiles * time per tile.  The times are the
+// measured ones of the solver's projector and backprojector (mean of both, 240^2 x
+// 512 and 160^2 x 48, 300 views, FP32) relative to the form {4, 1}; they follow
+// the 16-, 8- or 4-byte loads of a tap plus its fixed part.  E.g. 160^2 x 160,
+// projector: {2, 3} 0.098 ms, {4, 2} 0.113, {4, 1} 0.152.  Double precision
+// keeps two forms of pairs, and single values up to nz = 32, where pairs leave
+// half of the lanes idle (200^2 x 16: 2.70 ms, single 1.81).
+template <typename C, typename F>
+inline void with_z_form(int nz, int gmax, F&& f) {
+  if constexpr (sizeof(C) == 8) {
+    if (gmax >= 2 && nz % 128 == 0) f(ZForm<2, 2, false>{});
+    else if (gmax >= 2 && nz > 32) f(ZForm<2, 1, true>{});
+    else f(ZForm<1, 1, true>{});
+  } else {
+    if (gmax >= 4 && nz % 256 == 0) return f(ZForm<4, 2, false>{});
+    struct Cost { int G, NG; double time; };
+    constexpr Cost forms[10] = {{4, 2, 1.5}, {4, 1, 1.0}, {2, 4, 1.63}, {2, 3, 1.3}, {2, 2, 1.09},
+                                {2, 1, 0.87}, {1, 8, 2.2}, {1, 4, 1.17}, {1, 2, 0.96}, {1, 1, 0.76}};
+    int best = 9;
+    double least = 1e300;
+    for (int i = 0; i < 10; ++i) {
+      const int T = 32 * forms[i].G * forms[i].NG;
+      const double cost = ((nz + T - 1) / T) * forms[i].time;
+      if (forms[i].G <= gmax && cost < least) { least = cost; best = i; }
+    }
+    switch (best) {
+      case 0: return f(ZForm<4, 2, true>{});
+      case 1: return f(ZForm<4, 1, true>{});
+      case 2: return f(ZForm<2, 4, true>{});
+      case 3: return f(ZForm<2, 3, true>{});
+      case 4: return f(ZForm<2, 2, true>{});
+      case 5: return f(ZForm<2, 1, true>{});
+      case 6: return f(ZForm<1, 8, true>{});
+      case 7: return f(ZForm<1, 4, true>{});
+      case 8: return f(ZForm<1, 2, true>{});
+      default: return f(ZForm<1, 1, true>{});
+    }
+  }
 }
 
 }  // namespace sipo

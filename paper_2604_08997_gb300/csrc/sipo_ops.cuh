@@ -92,6 +92,7 @@ struct NeedBits {
   const uint32_t* rows;  // nullptr: use the vial spans instead
   const uint32_t* cols;
   int wr, wc;            // words per row / per column
+  bool spread;           // flags dilated by a PSF (may lie outside the vial)
   __device__ __forceinline__ unsigned window(const uint32_t* base, int line, int start) const {
     const int w = base == rows ? wr : wc;
     int b = start + kNbPad;
@@ -184,9 +185,11 @@ __device__ __forceinline__ void fma_z(C (&acc)[ZL], C w, const C (&v)[ZL]) {
   }
 }
 
-template <bool ROWS, bool FAST, typename SI, typename C, int ZL>
+template <bool ROWS, bool FAST, typename Z, typename SI, typename C>
 __device__ __forceinline__ void fp_walk(const Geo<C>& g, const SI* vz, const NeedBits& nb, bool use_bits, int k,
-                                        C jf, C c, C s, int lo, int hi, TapList<C>& tl, C (&acc)[ZL]) {
+                                        C jf, C c, C s, int lo, int hi, const ZSpan<Z>& zs, TapList<C>& tl,
+                                        C (&acc)[Z::ZL]) {
+  constexpr int ZL = Z::ZL;
   const int lane = threadIdx.x & 31;
   const C a = ROWS ? c : s;
   const C inv_a = C(1) / a, h = C(1) / fabs(a) + C(kCandEps);
@@ -222,13 +225,13 @@ __device__ __forceinline__ void fp_walk(const Geo<C>& g, const SI* vz, const Nee
     for (; t + 4 <= total; t += 4) {
       C v[4][ZL];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) load_z<SI, C, ZL>(vz + (size_t)tl.col[t + u] * g.nz, v[u]);
+      for (int u = 0; u < 4; ++u) load_zf<Z>(vz + (size_t)tl.col[t + u] * g.nz, zs, v[u]);
 #pragma unroll
       for (int u = 0; u < 4; ++u) fma_z<C, ZL>(acc, tl.w[t + u], v[u]);
     }
     for (; t < total; ++t) {
       C v[ZL];
-      load_z<SI, C, ZL>(vz + (size_t)tl.col[t] * g.nz, v);
+      load_zf<Z>(vz + (size_t)tl.col[t] * g.nz, zs, v);
       fma_z<C, ZL>(acc, tl.w[t], v);
     }
     __syncwarp();
@@ -241,22 +244,23 @@ __host__ __device__ constexpr int fp_reductions(int mode) {
 }
 
 // What a projector mode does with a finished z-vector of rays (g = acc) at
-// element `base` (z index z0).
-template <typename S, typename C, int ZL, int MODE, typename O>
-__device__ __forceinline__ void fp_finish(const Bufs<S, C>& b, const StepScalars<C>& sc, O* out, size_t base, int z0,
-                                          const C (&acc)[ZL], double* red, unsigned long long* kz_block) {
+// element `base` (that of group 0).
+template <typename S, typename C, typename Z, int MODE, typename O>
+__device__ __forceinline__ void fp_finish(const Bufs<S, C>& b, const StepScalars<C>& sc, O* out, size_t base,
+                                          const ZSpan<Z>& zs, const C (&acc)[Z::ZL], double* red,
+                                          unsigned long long* kz_block) {
   if constexpr (MODE == kFpStore) {
-    store_z<O, C, ZL>(out + base, acc);
+    store_owned<Z>(out + base, zs, acc);
   } else if constexpr (MODE == kFpPrimal) {
-    primal_update<S, C, ZL, false>(b, sc, base, acc, red);
+    primal_update<S, C, Z, false>(b, sc, base, zs, acc, red);
   } else if constexpr (MODE == kFpPrimalCheck) {
-    primal_update<S, C, ZL, true>(b, sc, base, acc, red);
+    primal_update<S, C, Z, true>(b, sc, base, zs, acc, red);
   } else if constexpr (MODE == kFpResid) {
-    resid_update<S, C, ZL>(b, base, acc, red);
+    resid_update<S, C, Z>(b, base, zs, acc, red);
   } else if constexpr (MODE == kFpCert) {
-    cert_update<S, C, ZL>(b, base, acc, red);
+    cert_update<S, C, Z>(b, base, zs, acc, red);
   } else {
-    cert_update_z<S, C, ZL>(b, base, z0, acc, kz_block);
+    cert_update_z<S, C, Z>(b, base, zs, acc, kz_block);
   }
 }
 
@@ -305,16 +309,16 @@ __device__ __forceinline__ void fp_ray_span(const Geo<C>& g, C sj, C c, C s, boo
 // and z group.  Rays of neighbouring views at one bin run almost on top of
 // each other, so a tile of 4 views x 2 bins meets more of its columns in L1
 // than 8 bins of one view (see launch_project for the measurements).
-template <typename SI, typename S, typename C, int ZL, int MODE, typename O>
+template <typename SI, typename S, typename C, typename Z, int MODE, typename O>
 __global__ void __launch_bounds__(kThreads, sizeof(C) == 8 ? 2 : 4)
 k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __restrict__ out,
           const uint8_t* __restrict__ act_col, const NeedBits nb, const int2* __restrict__ rspan, int aw) {
   const bool use_bits = nb.rows != nullptr;
   if (MODE != kFpStore && b.st->done) return;
-  constexpr int ZC = 32 * ZL;
+  constexpr int ZL = Z::ZL;
   constexpr int NR = fp_reductions(MODE);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nzc = (g.nz + ZC - 1) / ZC;
+  const int nzc = (g.nz + Z::T - 1) / Z::T;
   const int bw = kWarps / aw;
   const int njb = (g.nd + bw - 1) / bw, nka = (g.na + aw - 1) / aw;
   const long long ntiles = (long long)nka * njb * nzc;
@@ -336,21 +340,20 @@ k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __r
     const int tz = int(t1 % nzc);
     const int jb = int(t1 / nzc);
     const int j = jb * bw + warp / aw;
-    const int z0 = tz * ZC + lane * ZLayout<C, ZL>::G;
     if (aw > 1) __syncthreads();  // keeps the rays of a tile abreast, so that they meet in L1
     if (j >= g.nd || k >= g.na) continue;
     if (MODE != kFpStore && act_col != nullptr && !act_col[(size_t)k * g.nd + j]) continue;
+    ZSpan<Z> zs;
+    zs.init(g.nz, tz);
     const C esj = g.es ? g.es[(size_t)k * g.nd + j] : C(1);
     C acc[ZL];
 #pragma unroll
     for (int i = 0; i < ZL; ++i) acc[i] = C(0);
-    // The whole warp walks the ray (the walk uses warp shuffles); a lane past
-    // the end of a ragged z column reads the column's first group instead and
-    // never stores its result.
+    // The whole warp walks the ray (the walk uses warp shuffles).
     if (esj != C(0)) {
       const C c = g.cs[2 * k], s = g.cs[2 * k + 1];
       const C jf = C(j);
-      const SI* vz = vol + (z0 < g.nz ? z0 : 0);
+      const SI* vz = vol + zs.z0;
       const bool rows = fabs(c) >= fabs(s);
       int lo = 0, hi = (rows ? g.ny : g.nx) - 1;
       fp_ray_span<C>(g, jf - g.off, c, s, rows, lo, hi);
@@ -361,19 +364,18 @@ k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __r
       }
       TapList<C>& tl = taps[warp];
       if (rows) {
-        if (j >= 2) fp_walk<true, true, SI, C, ZL>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, tl, acc);
-        else fp_walk<true, false, SI, C, ZL>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, tl, acc);
+        if (j >= 2) fp_walk<true, true, Z, SI, C>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, zs, tl, acc);
+        else fp_walk<true, false, Z, SI, C>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, zs, tl, acc);
       } else {
-        if (j >= 2) fp_walk<false, true, SI, C, ZL>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, tl, acc);
-        else fp_walk<false, false, SI, C, ZL>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, tl, acc);
+        if (j >= 2) fp_walk<false, true, Z, SI, C>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, zs, tl, acc);
+        else fp_walk<false, false, Z, SI, C>(g, vz, nb, use_bits, k, jf, c, s, lo, hi, zs, tl, acc);
       }
 #pragma unroll
       for (int i = 0; i < ZL; ++i) acc[i] *= esj;
     }
-    if (z0 >= g.nz) continue;
-    const size_t base = ((size_t)k * g.nd + j) * g.nz + z0;
-    SIPO_DCHECK((z0 + z_offset<C, ZL>(ZL - 1) < g.nz), 0);
-    fp_finish<S, C, ZL, MODE, O>(b, sc, out, base, z0, acc, red, kz_block);
+    if (Z::kRagged && zs.fresh == 0u) continue;
+    SIPO_DCHECK(zs.z0 + zs.at(Z::NG - 1) + Z::G - 1 < g.nz, 0);
+    fp_finish<S, C, Z, MODE, O>(b, sc, out, ((size_t)k * g.nd + j) * g.nz + zs.z0, zs, acc, red, kz_block);
   }
   fp_reduce<MODE, kWarps>(g, b, red, kz_block, blockIdx.x < ntiles);
 }
@@ -591,20 +593,23 @@ k_backproject(const Geo<C> g, const SI* __restrict__ sino, const Bufs<S, C> b, O
 }
 
 // ------------------------------------------ backprojector with row patterns
-// Single-precision form of k_backproject with the same tiles, z layout,
-// angle order and epilogues, and sums equal bit for bit.  Per angle the lanes
-// write, for the warp's four voxels (x order), the first detector row
-// b = min floor(u), the offsets floor(u_v) - b packed two bits each (the
-// pattern) and the weights, each one twice (a float pair for the packed
-// multiply-add), with zero weight on every tap whose bin is off the detector.
-// u = fma(x, cos, inner) is monotone in x, so with |cos| <= 1 the offsets
-// move by 0 or 1 from one voxel to the next: 15 patterns.  Each pattern has a
-// body whose row indices are compile-time constants: the angle's two to five
-// rows are loaded at once into named registers, clamped to the detector (a
-// clamped row only meets zero weights, and 0 * x leaves a sum unchanged), and
-// every voxel applies its two rows with packed FP32 multiply-adds
-// (__ffma2_rn, two z values per instruction, each rounded like fmaf).  A
-// pattern outside the 15 takes a generic body that loads each voxel's rows.
+// Single-precision backprojector.  A warp owns four consecutive voxels of a row
+// and one z tile.  Per view the lanes write, for the four voxels (x order), the
+// first detector row b = min floor(u), the offsets floor(u_v) - b packed two
+// bits each (the pattern) and the weights, each one twice (a float pair for the
+// packed multiply-add), with zero weight on every tap whose bin is off the
+// detector.  u = fma(x, cos, inner) is monotone in x, so with |cos| <= 1 the
+// offsets move by 0 or 1 from one voxel to the next: 15 patterns.  Each pattern
+// has a body whose row indices are compile-time constants: the view's two to
+// five rows are loaded at once into named registers and every voxel applies its
+// two rows with packed FP32 multiply-adds (__ffma2_rn, two z values per
+// instruction, each rounded like fmaf).  Views whose rows run over an end of the
+// detector, and a pattern outside the 15, take a generic body that loads each
+// voxel's rows clamped (a clamped row only meets zero weights); views that miss
+// the detector with all four voxels are skipped.
+//
+// Bound: latency of the row loads first (24 warps an SM at 80 registers), then
+// L1 delivery (8.3 16-byte loads a lane per view at 8 z values, 4.1 taps a load).
 struct alignas(16) Bp2Ent {
   float4 w[4];  // voxel v: (w0, w0, w1, w1)
   int b, pat, pad0, pad1;
@@ -612,7 +617,17 @@ struct alignas(16) Bp2Ent {
 };
 constexpr int kBp2Chunk = 32;
 constexpr int kBp2Generic = 0xff;
+constexpr int kBp2Skip = 0xfe;
 constexpr int kBp2NV = 4;
+
+// Block tiles of k_backproject2: 8 >> split rows of 4 voxels, the views of a row
+// shared by 1 << split warps.  list: the tiles that hold a needed column, as
+// tile row * tiles per row + tile column (nullptr: every tile, n unused).
+struct BpTiles {
+  const int* list;
+  int n;
+  int split;
+};
 
 __host__ __device__ constexpr int bp2_off(int pat, int v) { return (pat >> (2 * v)) & 3; }
 __host__ __device__ constexpr int bp2_rows(int pat) {
@@ -621,7 +636,7 @@ __host__ __device__ constexpr int bp2_rows(int pat) {
   return m + 2;
 }
 
-__device__ __forceinline__ void bp2_fill(const Geo<float>& g, int k, float yf, float xf0, int iy, int tx0,
+__device__ __forceinline__ void bp2_weights(const Geo<float>& g, int k, float yf, float xf0, int iy, int tx0,
                                          unsigned mask, Bp2Ent& out) {
   const float c = g.cs[2 * k], s = g.cs[2 * k + 1];
   const float inner = geo_inner(yf, s, g.off);
@@ -674,6 +689,20 @@ __device__ __forceinline__ void bp2_fill(const Geo<float>& g, int k, float yf, f
   out.i0 = make_int4(i0[0], i0[1], i0[2], i0[3]);
 }
 
+// The entry for rows read in place: a patterned body reads all of its rows, b ..
+// b + top + 1, unclamped.
+__device__ __forceinline__ void bp2_fill(const Geo<float>& g, int k, float yf, float xf0, int iy, int tx0,
+                                         unsigned mask, Bp2Ent& out) {
+  Bp2Ent e;
+  bp2_weights(g, k, yf, xf0, iy, tx0, mask, e);
+  bool on = false;
+#pragma unroll
+  for (int v = 0; v < kBp2NV; ++v) on = on || e.w[v].x != 0.0f || e.w[v].z != 0.0f;
+  const int top = max(max(e.i0.x, e.i0.y), max(e.i0.z, e.i0.w)) + 1;
+  if (e.pat == kBp2Generic || e.b < 0 || top >= g.nd) e.pat = on ? kBp2Generic : kBp2Skip;
+  out = e;
+}
+
 // acc += w0 * r0 + w1 * r1 elementwise (w0 applied first), packed in pairs.
 template <int ZL>
 __device__ __forceinline__ void bp2_fma(float (&acc)[ZL], const float4& w, const float (&r0)[ZL],
@@ -694,33 +723,29 @@ __device__ __forceinline__ void bp2_fma(float (&acc)[ZL], const float4& w, const
   }
 }
 
-template <typename SI, int ZL>
-__device__ __forceinline__ void bp2_row(const Geo<float>& g, const SI* srow, int r, float (&t)[ZL]) {
-  r = r < 0 ? 0 : (r >= g.nd ? g.nd - 1 : r);
-  load_z<SI, float, ZL>(srow + (size_t)r * g.nz, t);
-}
-
-template <typename SI, int ZL, int PAT>
-__device__ __forceinline__ void bp2_body(const Geo<float>& g, const SI* srow, const Bp2Ent& e,
-                                         float (&acc)[kBp2NV][ZL]) {
+// The rows of one view, in place (srow: the lane's first element of bin 0).
+template <typename Z, typename SI, int PAT>
+__device__ __forceinline__ void bp2_body(const SI* row, size_t stride, const ZSpan<Z>& zs, const Bp2Ent& e,
+                                         float (&acc)[kBp2NV][Z::ZL]) {
   constexpr int NR = bp2_rows(PAT);
-  float r[NR][ZL];
+  float r[NR][Z::ZL];
 #pragma unroll
-  for (int j = 0; j < NR; ++j) bp2_row<SI, ZL>(g, srow, e.b + j, r[j]);
+  for (int j = 0; j < NR; ++j) load_zf<Z>(row + j * stride, zs, r[j]);
 #pragma unroll
-  for (int v = 0; v < kBp2NV; ++v) bp2_fma<ZL>(acc[v], e.w[v], r[bp2_off(PAT, v)], r[bp2_off(PAT, v) + 1]);
+  for (int v = 0; v < kBp2NV; ++v)
+    bp2_fma<Z::ZL>(acc[v], e.w[v], r[bp2_off(PAT, v)], r[bp2_off(PAT, v) + 1]);
 }
 
-template <typename SI, int ZL>
-__device__ __forceinline__ void bp2_generic(const Geo<float>& g, const SI* srow, const Bp2Ent& e,
-                                         float (&acc)[kBp2NV][ZL]) {
+template <typename Z, typename SI>
+__device__ __forceinline__ void bp2_generic(const SI* srow, size_t stride, int nd, const ZSpan<Z>& zs,
+                                            const Bp2Ent& e, float (&acc)[kBp2NV][Z::ZL]) {
   const int i0[kBp2NV] = {e.i0.x, e.i0.y, e.i0.z, e.i0.w};
 #pragma unroll
   for (int v = 0; v < kBp2NV; ++v) {
-    float r0[ZL], r1[ZL];
-    bp2_row<SI, ZL>(g, srow, i0[v], r0);
-    bp2_row<SI, ZL>(g, srow, i0[v] + 1, r1);
-    bp2_fma<ZL>(acc[v], e.w[v], r0, r1);
+    float r0[Z::ZL], r1[Z::ZL];
+    load_zf<Z>(srow + min(max(i0[v], 0), nd - 1) * stride, zs, r0);
+    load_zf<Z>(srow + min(max(i0[v] + 1, 0), nd - 1) * stride, zs, r1);
+    bp2_fma<Z::ZL>(acc[v], e.w[v], r0, r1);
   }
 }
 
@@ -728,119 +753,133 @@ __device__ __forceinline__ void bp2_generic(const Geo<float>& g, const SI* srow,
   X(0x00) X(0x40) X(0x50) X(0x90) X(0x54) X(0x94) X(0xA4) X(0xE4)                          \
   X(0x01) X(0x05) X(0x15) X(0x06) X(0x16) X(0x1A) X(0x1B)
 
-// One angle of a warp's four voxels: dispatch on the table entry's pattern.
-template <typename SI, int ZL>
-__device__ __forceinline__ void bp2_angle(const Geo<float>& g, const SI* srow, const Bp2Ent& e,
-                                          float (&acc)[kBp2NV][ZL]) {
+// One view of a warp's four voxels: dispatch on the table entry's pattern.
+template <typename Z, typename SI>
+__device__ __forceinline__ void bp2_angle(const SI* srow, size_t stride, int nd, const ZSpan<Z>& zs,
+                                          const Bp2Ent& e, float (&acc)[kBp2NV][Z::ZL]) {
+  const SI* row = srow + e.b * stride;
   switch (e.pat) {
 #define SIPO_BP2_CASE(P) \
   case P:                \
-    bp2_body<SI, ZL, P>(g, srow, e, acc); break;
+    bp2_body<Z, SI, P>(row, stride, zs, e, acc); break;
     SIPO_BP2_PATTERNS(SIPO_BP2_CASE)
 #undef SIPO_BP2_CASE
+    case kBp2Skip: break;
     default:
-      bp2_generic<SI, ZL>(g, srow, e, acc);
+      bp2_generic<Z, SI>(srow, stride, nd, zs, e, acc);
   }
 }
 
-// Tile: 4 voxel columns along x per warp, one row per warp (8 rows per
-// block), ZL z values per lane; need, modes and epilogues as in
-// k_backproject.
-template <typename SI, typename S, int ZL, int MINB, int MODE, typename O>
+// need, modes and epilogues as in k_backproject.  Each warp sums its share of the
+// views (a contiguous range, increasing); the shares of a voxel are added in
+// order and finished from shared memory, the groups of a row dealt out to its
+// warps.
+template <typename SI, typename S, typename Z, int MINB, int MODE, typename O>
 __global__ void __launch_bounds__(kThreads, MINB)
 k_backproject2(const Geo<float> g, const SI* __restrict__ sino, const Bufs<S, float> b, O* __restrict__ out,
-               const uint8_t* __restrict__ need) {
+               const uint8_t* __restrict__ need, const BpTiles tiles) {
   using C = float;
-  constexpr int NV = kBp2NV;
+  constexpr int NV = kBp2NV, G = Z::G, NG = Z::NG;
   if (MODE != kBpStore && b.st->done) return;
-  constexpr int ZC = 32 * ZL;
   constexpr int NR = MODE == kBpDual ? 2 : 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ntx = (g.nx + NV - 1) / NV, nty = (g.ny + kWarps - 1) / kWarps;
-  const int nzc = (g.nz + ZC - 1) / ZC;
-  const long long ntiles = (long long)ntx * nty * nzc;
+  const int nsplit = 1 << tiles.split, nrow = kWarps >> tiles.split;
+  const int ntx = (g.nx + NV - 1) / NV, nty = (g.ny + nrow - 1) / nrow;
+  const int nzc = (g.nz + Z::T - 1) / Z::T;
+  const long long ntiles = (tiles.list ? (long long)tiles.n : (long long)ntx * nty) * nzc;
   double red[NR > 0 ? NR : 1] = {};
   StepScalars<C> sc{};
   if (MODE != kBpStore) sc = read_scalars<C>(b.st);
+  // per warp: the view table, then the accumulators [voxel][group][lane][G]
   constexpr size_t kTableBytes = sizeof(Bp2Ent) * kBp2Chunk;
-  constexpr size_t kStageBytes = size_t(NV) * ZL * 32 * sizeof(C);
-  constexpr bool kStage = MODE != kBpStore && kStageBytes <= 4096;
-  constexpr size_t kWarpBytes = kTableBytes > (kStage ? kStageBytes : 0) ? kTableBytes : kStageBytes;
+  constexpr size_t kStageBytes = size_t(NV) * Z::ZL * 32 * sizeof(C);
+  constexpr size_t kWarpBytes = kTableBytes > kStageBytes ? kTableBytes : kStageBytes;
   __shared__ __align__(16) unsigned char smem_warp[kWarps][kWarpBytes];
   Bp2Ent* tb = reinterpret_cast<Bp2Ent*>(smem_warp[warp]);
+  const int ag = warp & (nsplit - 1);
+  const int k_lo = int((long long)g.na * ag / nsplit), k_hi = int((long long)g.na * (ag + 1) / nsplit);
+  const size_t stride = g.nz;
 
   for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int tz = int(t % nzc);
-    const long long t1 = t / nzc;
-    const int tx = int(t1 % ntx);
-    const int ty = int(t1 / ntx);
-    const int iy = ty * kWarps + warp;
-    const int z0 = tz * ZC + lane * ZLayout<C, ZL>::G;
-    if (iy >= g.ny) continue;
-    const int2 sp = g.xspan[iy];
+    const int tile = tiles.list ? tiles.list[t / nzc] : int(t / nzc);
+    const int tx = tile % ntx, iy = tile / ntx * nrow + (warp >> tiles.split);
     unsigned mask = 0;
+    if (iy < g.ny) {
+      const int2 sp = g.xspan[iy];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int ix = tx * NV + v;
-      if (ix < g.nx && ix >= sp.x && ix <= sp.y && (need == nullptr || need[(size_t)iy * g.nx + ix]))
-        mask |= 1u << v;
+      for (int v = 0; v < NV; ++v) {
+        const int ix = tx * NV + v;
+        if (ix < g.nx && ix >= sp.x && ix <= sp.y && (need == nullptr || need[(size_t)iy * g.nx + ix]))
+          mask |= 1u << v;
+      }
     }
-    C acc[NV][ZL];
+    ZSpan<Z> zs;
+    zs.init(g.nz, tz);
+    C acc[NV][Z::ZL];
 #pragma unroll
     for (int v = 0; v < NV; ++v)
 #pragma unroll
-      for (int i = 0; i < ZL; ++i) acc[v][i] = C(0);
-    // the whole warp takes part; a lane past the end of a ragged z column
-    // reads the column's first group and never stores its result
+      for (int i = 0; i < Z::ZL; ++i) acc[v][i] = C(0);
     if (mask != 0u) {
       const C yf = C(iy) - g.cy;
       const C xf0 = C(tx * NV) - g.cx;
-      const SI* sz = sino + (z0 < g.nz ? z0 : 0);
-      for (int k0 = 0; k0 < g.na; k0 += kBp2Chunk) {
-        if (k0 + lane < g.na) bp2_fill(g, k0 + lane, yf, xf0, iy, tx * NV, mask, tb[lane]);
+      const SI* srow = sino + zs.z0 + (size_t)k_lo * g.nd * stride;
+      for (int k0 = k_lo; k0 < k_hi; k0 += kBp2Chunk) {
+        if (k0 + lane < k_hi) bp2_fill(g, k0 + lane, yf, xf0, iy, tx * NV, mask, tb[lane]);
         __syncwarp();
-        const int kn = min(kBp2Chunk, g.na - k0);
-        for (int kk = 0; kk < kn; ++kk)
-          bp2_angle<SI, ZL>(g, sz + (size_t)(k0 + kk) * g.nd * g.nz, tb[kk], acc);
+        const int kn = min(kBp2Chunk, k_hi - k0);
+        for (int kk = 0; kk < kn; ++kk, srow += g.nd * stride)
+          bp2_angle<Z, SI>(srow, stride, g.nd, zs, tb[kk], acc);
         __syncwarp();
       }
     }
-    using LS = ZLayout<C, ZL>;
-    C* stage = reinterpret_cast<C*>(smem_warp[warp]);
-    if constexpr (kStage) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int q = 0; q < LS::NG; ++q)
-#pragma unroll
-          for (int i = 0; i < LS::G; ++i) stage[((v * LS::NG + q) * 32 + lane) * LS::G + i] = acc[v][q * LS::G + i];
-      __syncwarp();
-    }
-    if (z0 >= g.nz) {
-      __syncwarp();
-      continue;
-    }
-    SIPO_DCHECK((z0 + z_offset<C, ZL>(ZL - 1) < g.nz), 2);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int ix = tx * NV + v;
-      if (ix >= g.nx) continue;
-      const size_t base = ((size_t)iy * g.nx + ix) * g.nz + z0;
+    const size_t base = ((size_t)iy * g.nx + tx * NV) * g.nz + zs.z0;
+    SIPO_DCHECK(zs.z0 + zs.at(NG - 1) + G - 1 < g.nz, 2);
+    if (MODE == kBpStore && nsplit == 1) {
       if constexpr (MODE == kBpStore) {
-        if (need == nullptr || ((mask >> v) & 1u)) store_z<O, C, ZL>(out + base, acc[v]);
-      } else if ((mask >> v) & 1u) {
-        using L = ZLayout<C, ZL>;
+        if (iy < g.ny) {
 #pragma unroll
-        for (int q = 0; q < L::NG; ++q) {
-          C part[L::G];
-#pragma unroll
-          for (int i = 0; i < L::G; ++i)
-            part[i] = kStage ? stage[((v * L::NG + q) * 32 + lane) * L::G + i] : acc[v][q * L::G + i];
-          dual_update<S, C, L::G, false>(b, sc, base + q * L::kStride, part, red);
+          for (int v = 0; v < NV; ++v)
+            if (tx * NV + v < g.nx && (need == nullptr || ((mask >> v) & 1u)))
+              store_owned<Z>(out + base + (size_t)v * g.nz, zs, acc[v]);
         }
       }
+      continue;
     }
-    __syncwarp();
+    C* stage = reinterpret_cast<C*>(smem_warp[warp]);
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+      for (int q = 0; q < NG; ++q)
+#pragma unroll
+        for (int i = 0; i < G; ++i) stage[((v * NG + q) * 32 + lane) * G + i] = acc[v][q * G + i];
+    if (nsplit > 1) __syncthreads();
+    else __syncwarp();
+    if (iy < g.ny) {
+      // the epilogue runs group by group to keep its live range short
+      const C* first = reinterpret_cast<const C*>(smem_warp[warp - ag]);
+#pragma unroll 1
+      for (int u = ag; u < NV * NG; u += nsplit) {
+        const int v = u / NG, q = u % NG;
+        const bool mine = tx * NV + v < g.nx && ((mask >> v) & 1u || (MODE == kBpStore && need == nullptr));
+        if (!mine || !((zs.fresh >> q) & 1u)) continue;
+        const int off = Z::kRagged ? min(q * 32 * G, max(g.nz - 32 * G, 0)) : q * 32 * G;
+        C part[G];
+#pragma unroll
+        for (int i = 0; i < G; ++i) part[i] = first[(u * 32 + lane) * G + i];
+        for (int a = 1; a < nsplit; ++a) {
+          const C* other = first + a * (kWarpBytes / sizeof(C));
+#pragma unroll
+          for (int i = 0; i < G; ++i) part[i] += other[(u * 32 + lane) * G + i];
+        }
+        const size_t at = base + (size_t)v * g.nz + off;
+        if constexpr (MODE == kBpStore) store_group<O, C, G>(out + at, part);
+        else dual_update<S, C, G, false>(b, sc, at, part, red);
+      }
+    }
+    if (nsplit > 1) __syncthreads();
+    else __syncwarp();
   }
   if constexpr (MODE == kBpDual) block_reduce_store<2>(red, b.part, kSlSBand, blockIdx.x < ntiles);
 }

@@ -46,27 +46,27 @@ __global__ void k_need_bits(const uint8_t* __restrict__ need, uint32_t* __restri
 
 template <typename SI, typename S, typename C, int MODE, typename O>
 void launch_project(const Geo<C>& g, const SI* vol, const Bufs<S, C>& b, O* out,
-                    const uint8_t* act_col, int zl, cudaStream_t stream, const NeedBits& nb,
+                    const uint8_t* act_col, cudaStream_t stream, const NeedBits& nb,
                     const int2* rspan) {
-  constexpr int G = z_group<C>();
   // the slice-mode certificate keeps one 8-byte maximum per z in shared memory
   const size_t dyn = MODE == kFpCertZ ? size_t(g.nz) * sizeof(unsigned long long) : 0;
-  if (zl == 1 && g.nz <= kFlatMaxZ) {
-    k_project_flat<SI, S, C, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, rspan);
+  if (fp_flat<C>(g.nz)) {
+    // a solver's input vanishes outside its flagged columns; those may lie
+    // outside the vial where a PSF spreads them
+    const bool wide = nb.rows != nullptr && g.r2i >= 0 && nb.spread;
+    k_project_flat<SI, S, C, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, rspan, wide);
     return;
   }
-  // Views per tile: 4 where every block has several tiles to even out, else 1.
-  // 256^3 x 360 (9.5 tiles a block), solver step: 0.420 ms with 1, 0.394 with 2,
-  // 0.360 with 4, 0.364 with 8 (another target: 0.704, 0.605, 0.616, 0.655);
-  // 96^3 x 391 (4 tiles a block): 0.067 ms with 1, 0.072 with 4.
-  const long long tiles = (long long)g.na * ((g.nd + kWarps - 1) / kWarps) * ((g.nz + 32 * zl - 1) / (32 * zl));
-  const int aw = tiles >= 8LL * kRedBlocks ? 4 : 1;
-  if (zl == 2 * G)
-    k_project<SI, S, C, 2 * G, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan, aw);
-  else if (zl == G)
-    k_project<SI, S, C, G, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan, aw);
-  else
-    k_project<SI, S, C, 1, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan, aw);
+  with_z_form<C>(g.nz, z_group_for<C>(g.nz, vol, out), [&](auto form) {
+    using Z = decltype(form);
+    // Views per tile: 4 where every block has several tiles to even out, else 1.
+    // 256^3 x 360 (9.5 tiles a block), solver step: 0.420 ms with 1, 0.394 with 2,
+    // 0.360 with 4, 0.364 with 8 (another target: 0.704, 0.605, 0.616, 0.655);
+    // 96^3 x 391 (4 tiles a block): 0.067 ms with 1, 0.072 with 4.
+    const long long tiles = (long long)g.na * ((g.nd + kWarps - 1) / kWarps) * ((g.nz + Z::T - 1) / Z::T);
+    const int aw = tiles >= 8LL * kRedBlocks ? 4 : 1;
+    k_project<SI, S, C, Z, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan, aw);
+  });
 }
 
 void launch_need_bits(const uint8_t* need, uint32_t* rows, uint32_t* cols, int nx, int ny, int wr, int wc,
@@ -88,7 +88,7 @@ template void launch_ray_spans<double>(const Geo<double>&, const uint8_t*, int2*
 
 #define SIPO_FP(SI, S, C, M, O) \
   template void launch_project<SI, S, C, M, O>(const Geo<C>&, const SI*, const Bufs<S, C>&, O*, \
-                                                const uint8_t*, int, cudaStream_t, const NeedBits&, \
+                                                const uint8_t*, cudaStream_t, const NeedBits&, \
                                                 const int2*);
 #define SIPO_FP_SOLVER(S, C)          \
   SIPO_FP(S, S, C, kFpPrimal, C)      \

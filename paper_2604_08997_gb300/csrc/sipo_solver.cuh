@@ -291,17 +291,18 @@ __device__ __forceinline__ void dual_update(const Bufs<S, C>& b, const StepScala
 // ----------------------------------------------------------- primal update
 // One z-vector of rays with g = A q already formed.  CHECK = false: Halpern
 // step fused; CHECK = true: writes y+ and the restart distances (red[0..1]).
-template <typename S, typename C, int ZL, bool CHECK>
-__device__ __forceinline__ void primal_update(const Bufs<S, C>& b, const StepScalars<C>& sc,
-                                              size_t base, const C (&g)[ZL], double* red) {
+template <typename S, typename C, typename Z, bool CHECK>
+__device__ __forceinline__ void primal_update(const Bufs<S, C>& b, const StepScalars<C>& sc, size_t base,
+                                              const ZSpan<Z>& zs, const C (&g)[Z::ZL], double* red) {
+  constexpr int ZL = Z::ZL;
   C col[ZL], y[ZL], y0[ZL], yb[ZL], yo[ZL];
-  load_z<C, C, ZL>(b.col + base, col);
+  load_owned<Z>(b.col + base, zs, col);
   bool any = false;
 #pragma unroll
   for (int i = 0; i < ZL; ++i) any |= col[i] > C(0);
   if (!any) return;  // every ray of the vector is masked: y, y_bar stay 0
-  load_z<S, C, ZL>(b.y + base, y);
-  load_z<S, C, ZL>(b.y0 + base, y0);
+  load_owned<Z>(b.y + base, zs, y);
+  load_owned<Z>(b.y0 + base, zs, y0);
   const C w = sc.w;
   C a0 = C(0), a1 = C(0);  // restart distances of this z-vector (compute type)
 #pragma unroll
@@ -323,22 +324,24 @@ __device__ __forceinline__ void primal_update(const Bufs<S, C>& b, const StepSca
     red[0] += double(a0);
     red[1] += double(a1);
   }
-  store_z<S, C, ZL>(b.ybar + base, yb);
+  store_owned<Z>(b.ybar + base, zs, yb);
   if constexpr (!CHECK) {
-    store_z<S, C, ZL>(b.y + base, yo);
+    store_owned<Z>(b.y + base, zs, yo);
   } else {
-    store_z<S, C, ZL>(b.yp + base, yo);
-    store_z<C, C, ZL>(b.gc + base, g);
+    store_owned<Z>(b.yp + base, zs, yo);
+    store_owned<Z>(b.gc + base, zs, g);
   }
 }
 
 // Bound-based certificate: largest max(-g^, 0) / b over active rays (red[0];
 // +inf where a violated ray has b = 0).
-template <typename S, typename C, int ZL>
-__device__ __forceinline__ void cert_update(const Bufs<S, C>& b, size_t base, const C (&g)[ZL], double* red) {
+template <typename S, typename C, typename Z>
+__device__ __forceinline__ void cert_update(const Bufs<S, C>& b, size_t base, const ZSpan<Z>& zs,
+                                            const C (&g)[Z::ZL], double* red) {
+  constexpr int ZL = Z::ZL;
   C col[ZL], bb[ZL];
-  load_z<C, C, ZL>(b.col + base, col);
-  load_z<C, C, ZL>(b.cert_b + base, bb);
+  load_owned<Z>(b.col + base, zs, col);  // (0 where not owned: skipped below)
+  load_owned<Z>(b.cert_b + base, zs, bb);
 #pragma unroll
   for (int i = 0; i < ZL; ++i) {
     if (col[i] > C(0) && g[i] < C(0)) {
@@ -353,29 +356,31 @@ __device__ __forceinline__ void cert_update(const Bufs<S, C>& b, size_t base, co
 // the block's shared array kz[nz] (the bit patterns of non-negative doubles,
 // +inf included, order like the values, so the maximum does not depend on
 // the order of the updates).
-template <typename S, typename C, int ZL>
-__device__ __forceinline__ void cert_update_z(const Bufs<S, C>& b, size_t base, int z0, const C (&g)[ZL],
-                                              unsigned long long* kz) {
+template <typename S, typename C, typename Z>
+__device__ __forceinline__ void cert_update_z(const Bufs<S, C>& b, size_t base, const ZSpan<Z>& zs,
+                                              const C (&g)[Z::ZL], unsigned long long* kz) {
+  constexpr int ZL = Z::ZL;
   C col[ZL], bb[ZL];
-  load_z<C, C, ZL>(b.col + base, col);
-  load_z<C, C, ZL>(b.cert_b + base, bb);
+  load_owned<Z>(b.col + base, zs, col);
+  load_owned<Z>(b.cert_b + base, zs, bb);
 #pragma unroll
   for (int i = 0; i < ZL; ++i) {
     if (col[i] > C(0) && g[i] < C(0)) {
       const double v = bb[i] > C(0) ? double(-g[i] / bb[i]) : CUDART_INF;
-      atomicMax(kz + z0 + z_offset<C, ZL>(i), (unsigned long long)__double_as_longlong(v));
+      atomicMax(kz + zs.z0 + zs.at(i / Z::G) + i % Z::G, (unsigned long long)__double_as_longlong(v));
     }
   }
 }
 
 // Dual residual of T(z) on active rays from g+ = A q+ (red[0..3]).
-template <typename S, typename C, int ZL>
-__device__ __forceinline__ void resid_update(const Bufs<S, C>& b, size_t base, const C (&g)[ZL],
-                                             double* red) {
+template <typename S, typename C, typename Z>
+__device__ __forceinline__ void resid_update(const Bufs<S, C>& b, size_t base, const ZSpan<Z>& zs,
+                                             const C (&g)[Z::ZL], double* red) {
+  constexpr int ZL = Z::ZL;
   C col[ZL], g0[ZL], gc[ZL];
-  load_z<C, C, ZL>(b.col + base, col);
-  load_z<C, C, ZL>(b.g0 + base, g0);
-  load_z<C, C, ZL>(b.gc + base, gc);
+  load_owned<Z>(b.col + base, zs, col);
+  load_owned<Z>(b.g0 + base, zs, g0);
+  load_owned<Z>(b.gc + base, zs, gc);
   // sums of one z-vector in the compute type, folded into FP64 once per
   // vector (as in the check-step dual update)
   C a0 = C(0), a1 = C(0), a2 = -CUDART_INF_F, a3 = -CUDART_INF_F;
@@ -394,7 +399,7 @@ __device__ __forceinline__ void resid_update(const Bufs<S, C>& b, size_t base, c
   red[1] += double(a1);
   red[2] = fmax(red[2], double(a2));
   red[3] = fmax(red[3], double(a3));
-  store_z<C, C, ZL>(b.gp + base, g);
+  store_owned<Z>(b.gp + base, zs, g);
 }
 
 }  // namespace sipo
