@@ -244,8 +244,9 @@ int sipo_response_metrics(sipo_ctx *ctx, const sipo_response *M, const float *m_
  * res->cert_slice names the slice.  y_out (nullable) receives y*, the normalised
  * projection of Eq. 18, as [n_angles][n_det][nz] in FP32 (FP64 when storage
  * is SIPO_F64), host or device per y_location.  Blocks until done.  Errors:
- * INVALID_ARG, CUDA, NUMERIC (a check found NaN or infinite residuals, e.g.
- * from an infinite imported start); the context stays usable. */
+ * INVALID_ARG, CUDA, TIMEOUT (a bounded device-side wait of the staged
+ * backprojector gave up), NUMERIC (a check found NaN or infinite residuals,
+ * e.g. from an infinite imported start); the context stays usable. */
 int sipo_solve(sipo_ctx *ctx, void *y_out, int y_location, sipo_result *res);
 
 /* Warm start, for precision escalation (a reading of the mixed-precision
@@ -428,7 +429,9 @@ const char *sipo_phase_name(int i);
 /* Number of entries in the backprojector tile table (for sipo_tolerances.tile_cfg).
  * Single precision: the row-pattern kernel (4 voxel columns a warp, the rows of
  * each angle in registers, packed FP32 multiply-adds) at 2 blocks/SM (entries 0,
- * 1, 3) or 3 (2, 4, 5, 6).  FP64: 0 = 8 voxel columns per warp at 2 blocks/SM, 1 =
+ * 1, 3) or 3 (2, 4); 5, 6 = its form with the rows staged in shared memory by
+ * tensor-memory copies, where nz is a multiple of 4 and the part is large enough
+ * (else as 4).  FP64: 0 = 8 voxel columns per warp at 2 blocks/SM, 1 =
  * 4 columns at 2 blocks/SM, 2-6 = 4 columns at 3 blocks/SM.  Volumes of few z
  * values have one kernel for every entry.  Every entry gives the same sums bit
  * for bit within one precision. */

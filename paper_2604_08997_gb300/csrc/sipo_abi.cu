@@ -160,7 +160,7 @@ struct Solver final : SolverBase {
   int ze = 1;  // elements per thread of the element-wise kernels
   // block tiles of the single-precision backprojector: those with a needed
   // column (solver steps), and all (the plain operator)
-  BpTiles bpt{nullptr, 0, 0}, bpt_all{nullptr, 0, 0};
+  BpTiles bpt{nullptr, 0, 8, 0}, bpt_all{nullptr, 0, 8, 0};
   int P = 64;
   bool psf = false;
   int bp_nv = 0;     // backprojector tile table entry
@@ -240,8 +240,8 @@ struct Solver final : SolverBase {
     cp = *c;
     tol = *t;
     P = tol.check_every > 0 ? tol.check_every : 64;
-    // the element-wise kernels run over whole arrays, whatever nz is
-    ze = (V % z_group<C>() == 0 && SN % z_group<C>() == 0) ? z_group<C>() : 1;
+    // (sums of a value at a time where z columns are not whole groups)
+    ze = nz % z_group<C>() == 0 ? z_group<C>() : 1;
     if (s) {
       stream = s;
     } else {
@@ -437,6 +437,7 @@ struct Solver final : SolverBase {
     ck(cudaGetLastError(), "Farkas test");
     ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
     ck(cudaStreamSynchronize(stream), "Farkas test");
+    check_bp_fault();
     const int cert = h_st->cert;
     if (slice) *slice = cert ? h_st->cert_z : -1;
     init_state();
@@ -855,23 +856,22 @@ struct Solver final : SolverBase {
   }
 
   // ------------------------------------------------- backprojector tiles
-  // Tiles of k_backproject2 with a column in `cols` ([y][x] flags, host), for
-  // 8 >> split rows a tile.
-  std::vector<int> bp_tile_list(const std::vector<uint8_t>& cols, int split) const {
-    const int nrow = kWarps >> split, ntx = (nx + kBp2NV - 1) / kBp2NV, nty = (ny + nrow - 1) / nrow;
+  // Tiles of `rows` x 4 voxels with a column in `cols` ([y][x] flags, host).
+  std::vector<int> bp_tile_list(const std::vector<uint8_t>& cols, int rows) const {
+    const int ntx = (nx + kBp2NV - 1) / kBp2NV, nty = (ny + rows - 1) / rows;
     std::vector<int> list;
     for (int ty = 0; ty < nty; ++ty)
       for (int tx = 0; tx < ntx; ++tx) {
         bool any = false;
-        for (int y = ty * nrow; y < std::min(ny, (ty + 1) * nrow) && !any; ++y)
+        for (int y = ty * rows; y < std::min(ny, (ty + 1) * rows) && !any; ++y)
           for (int x = tx * kBp2NV; x < std::min(nx, (tx + 1) * kBp2NV) && !any; ++x) any = cols[size_t(y) * nx + x];
         if (any) list.push_back(ty * ntx + tx);
       }
     return list;
   }
 
-  // Chooses the view split (by shape and target alone, so that sums do not
-  // depend on timing) and lists the solver's tiles.
+  // Chooses the tiles by shape and target alone (sums do not depend on timing)
+  // and lists the solver's.
   void choose_bp_tiles() {
     if constexpr (sizeof(C) == 8) return;
     int T = 1;
@@ -880,22 +880,35 @@ struct Solver final : SolverBase {
     std::vector<uint8_t> cols(size_t(nx) * ny);
     ck(cudaMemcpyAsync(cols.data(), need, cols.size(), cudaMemcpyDeviceToHost, stream), "need");
     ck(cudaStreamSynchronize(stream), "need");
-    const long long want = (long long)(1.75 * device_sms() * 3);
-    std::vector<int> list;
-    for (bpt.split = 0;; ++bpt.split) {
-      list = bp_tile_list(cols, bpt.split);
-      if ((long long)list.size() * nzc >= want || bpt.split == 3) break;
+    // Tiles of 8 rows where they cover the SMs one and a half times, else of 2: a
+    // tile lasts as long as its views, and on a small part more of them, on more
+    // SMs, is what is left to gain.  Staged rows, solver step, ms with 8 / 4 / 2 rows
+    // (tiles of 8): 64^3 x 180 (41) 0.060 / 0.057 / 0.054; 112^3 x 333 (134) 0.111 /
+    // 0.103 / 0.101; 160^3 x 300 (164) 0.136 / 0.125 / 0.126; 192^3 x 300 (286) 0.158 /
+    // 0.247 / 0.241; 256^3 x 360 (490) 0.338 / 0.422 / 0.505.
+    const long long want = 3LL * device_sms() / 2;
+    std::vector<int> list = bp_tile_list(cols, 8);
+    if ((long long)list.size() * nzc < want) {
+      bpt.rows = 2;
+      list = bp_tile_list(cols, 2);
     }
     int* d = dalloc<int>(list.size());
     ck(cudaMemcpyAsync(d, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, stream), "tiles");
     ck(cudaStreamSynchronize(stream), "tiles");
     bpt.list = d;
     bpt.n = int(list.size());
+    // the plain operator: every tile, of which about `share` have work
     const double share = vial_r > 0 ? std::min(1.0, 3.14159265 * vial_r * vial_r / (double(nx) * ny)) : 1.0;
-    for (bpt_all.split = 0; bpt_all.split < 3; ++bpt_all.split) {
-      const int nrow = kWarps >> bpt_all.split;
-      const double tiles = share * ((nx + kBp2NV - 1) / kBp2NV) * ((ny + nrow - 1) / nrow) * double(nzc);
-      if (tiles >= double(want)) break;
+    auto tiles = [&](int rows) { return share * ((nx + kBp2NV - 1) / kBp2NV) * ((ny + rows - 1) / rows) * double(nzc); };
+    if (bp_staged(nz)) {
+      if (tiles(8) < double(want)) bpt_all.rows = 2;
+    } else {
+      // without staged rows the chain of a warp's views is long: shared by up to
+      // eight warps until there are 1.75 rounds of the 3 resident blocks an SM.
+      // 128^2 x 130 x 360 (122 tiles of 8 rows), solver step, ms by split 0, 1, 2, 3:
+      // 0.199, 0.116, 0.079, 0.087.
+      while (bpt_all.split < 3 && tiles(8 >> bpt_all.split) < 1.75 * 3 * device_sms()) ++bpt_all.split;
+      bpt_all.rows = 8 >> bpt_all.split;
     }
   }
 
@@ -1090,12 +1103,14 @@ struct Solver final : SolverBase {
       launch_project<C, C, C, kFpStore, C>(g, t1, Bufs<C, C>{}, col, nullptr, stream);
     }
     k_apply_mask<C><<<gs, kThreads, 0, stream>>>(col, mask, (long long)SN);
-    // row abs-sums of A^T over active rays: A^T 1_act = K P^T 1_act
+    // row abs-sums of A^T over active rays: A^T 1_act = K P^T 1_act, in the
+    // solver's order of views
+    const BpTiles whole{nullptr, 0, bpt.rows, 0};
     if (psf) {
-      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, t1, nullptr, stream, bpt_all);
+      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, t1, nullptr, stream, whole);
       psf3<C, C>(t1, row, t2, t3, -1, stream);
     } else {
-      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, row, nullptr, stream, bpt_all);
+      launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, row, nullptr, stream, whole);
     }
     (void)B;
     // setup sums
@@ -1208,6 +1223,12 @@ struct Solver final : SolverBase {
       return;
     }
     if (bp_flat<C>(nz)) return;  // no tiles to choose from
+    if (sizeof(C) == 4 && bp_staged(nz)) {
+      // staged rows were the fastest entry on every size measured (64^3 to 384^3,
+      // FP32 and BF16 storage: 0.60 to 0.97 of the best of entries 3 and 4)
+      bp_nv = 5;
+      return;
+    }
     const TileKey key{nx, ny, nz, na, nd, tol.storage, psf ? 1 : 0};
     {
       std::lock_guard<std::mutex> lock(g_tile_mutex);
@@ -1404,6 +1425,7 @@ struct Solver final : SolverBase {
   void finish_solve(void* y_out, int loc, sipo_result* res) override {
     ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
     ck(cudaStreamSynchronize(stream), "solve");
+    check_bp_fault();
     if (!h_st->done) {
       final_check();
       ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
@@ -1458,6 +1480,15 @@ struct Solver final : SolverBase {
     res->kernel_launches = launches;
     res->tile_cfg = bp_nv;
     res->cert_slice = h.status == 1 ? h.cert_z : -1;
+  }
+
+  // A bounded wait inside the staged backprojector gave up (bit 0), or a view's
+  // rows did not fit its box (bit 1): the sums of that launch are not valid, so
+  // the solve is an error.
+  void check_bp_fault() {
+    const unsigned int f = bp_fault_take();
+    if (f & 1u) fail(SIPO_ERR_TIMEOUT, "backprojector: a wait on a tensor-memory copy timed out");
+    if (f) fail(SIPO_ERR_NUMERIC, "backprojector: detector rows outside the staged box");
   }
 
   // copies n elements of S (converted to C) to out (host or device)

@@ -347,16 +347,17 @@ __device__ __forceinline__ void floor_split(double u, double& fl, int& i) {
 // active (the same for the whole block): false where the block had no tile and
 // every value is still zero; it then stores zeros without the FP64 shuffles,
 // which cost a small problem more than its work (1216 blocks, 2 FP64 lanes per
-// clock and SM).  WARPS = 1: only the first warp holds values.
+// clock and SM).  warps: the first warps of the block, which hold values.
 template <int N, unsigned MAXMASK = 0u, int WARPS = kWarps>
-__device__ __forceinline__ void block_reduce_store(double (&v)[N], double* part, int slot0, bool active = true) {
+__device__ __forceinline__ void block_reduce_store(double (&v)[N], double* part, int slot0, bool active = true,
+                                                   int warps = WARPS) {
   __shared__ double red[kWarps][N > 0 ? N : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (!active) {
     if (threadIdx.x < N) part[(slot0 + threadIdx.x) * kRedBlocks + blockIdx.x] = 0.0;
     return;
   }
-  if (warp < WARPS) {
+  if (warp < warps) {
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     double x = v[i];
@@ -374,7 +375,7 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[N], double* part,
     const bool mx = (MAXMASK >> threadIdx.x) & 1u;
     double s = red[0][threadIdx.x];
 #pragma unroll
-    for (int w = 1; w < WARPS; ++w) s = mx ? fmax(s, red[w][threadIdx.x]) : s + red[w][threadIdx.x];
+    for (int w = 1; w < warps; ++w) s = mx ? fmax(s, red[w][threadIdx.x]) : s + red[w][threadIdx.x];
     SIPO_DCHECK(isfinite(s) || (mx && s == CUDART_INF), 3);
     part[(slot0 + threadIdx.x) * kRedBlocks + blockIdx.x] = s;
   }

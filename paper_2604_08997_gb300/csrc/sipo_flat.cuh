@@ -5,18 +5,21 @@
 // value: 31 lanes idle there, and the work per weight is one multiply-add.
 // Here the lanes hold 32 neighbouring bins of a view (projector) or 32
 // neighbouring voxels of a row (backprojector) of one z slice instead, each
-// lane computing its own weights, and the eight warps of a block share a tile:
-// each sums every eighth chunk of lines (or every eighth view), and the first
-// warp adds the eight partial sums in order and runs the epilogue.  The weights
-// are those of the z-lane kernels bit for bit (same u, same rounding); the sums
-// differ from theirs only in order, which is fixed.
+// lane computing its own weights.  The weights are those of the z-lane kernels
+// bit for bit (same u, same rounding).
 //
-// Bound: instruction issue on the weights (about 50 per bin and line, 20 per
+// Single precision: every warp has a tile of its own and adds its terms in the
+// order of the z-lane kernels, so the sums are theirs bit for bit too (a solve
+// amplifies a change of order: up to 2e-5 in the duals of Case 2 after 64
+// iterations).  Double precision: the eight warps of a block share a tile, each
+// summing every eighth chunk of lines (or every eighth view), and the first warp
+// adds the eight partial sums in order.
+//
+// Bound: instruction issue on the weights (about 55 per bin and line, 20 per
 // voxel and view), not bytes: a 512 x 512 slice and its 360 x 512 sinogram stay
-// in L2.  512 x 512, 360 views, single precision: projector 0.18 ms and
-// backprojector 0.06 ms, where the z-lane kernels took 5.4 ms for the pair; 64 x
-// 64, 96 views, double precision: 0.06 ms for the pair (0.25 ms), bound by FP64
-// issue.
+// in L2.  512 x 512, 360 views, single precision: 0.34 ms for a projection and a
+// backprojection, where the z-lane kernels took 5.4 ms; 64 x 64, 96 views, double
+// precision: 0.06 ms for the pair (0.25 ms), bound by FP64 issue.
 #pragma once
 
 #include "sipo_ops.cuh"
@@ -53,9 +56,11 @@ __device__ __forceinline__ bool flat_hit(float w) { return __float_as_uint(w) < 
 __device__ __forceinline__ bool flat_hit(double w) { return unsigned(__double2hiint(w)) < 0x3ff00000u; }
 
 // Sums of one lane's bin j over the warp's chunks of lines: each voxel with
-// floor(u) = j gives (1 - w) v to bin j (own) and w v to bin j + 1 (next), the
+// floor(u) = j gives (1 - w) v to bin j and w v to bin j + 1, the
 // backprojector's two taps, so that a voxel is read and weighed once for both
-// bins.  ROWS: the ray is walked along y (lines are rows, read from global
+// bins.  Single precision: `own` takes this lane's voxels and those of the lane
+// below (by shuffles), in increasing index along the line, like the per-ray walk;
+// double precision: `next` collects w v and moves up at the end.  ROWS: the ray is walked along y (lines are rows, read from global
 // memory: the lanes' voxels are neighbours along x); otherwise along x, the
 // chunk's columns staged in shared memory with reads along x.  EDGE: any tile
 // (bin -1 among its bins, any z stride, inputs that reach outside the vial);
@@ -75,7 +80,9 @@ __device__ __forceinline__ void flat_walk(const Geo<C>& g, const SI* vz, int k, 
   const float slope = float(-(ROWS ? s : c) * inv_a);
   const float base = float((jf - g.off + (ROWS ? g.cy * s : g.cx * c)) * inv_a + (ROWS ? g.cx : g.cy) +
                            (inv_a < C(0) ? inv_a : C(0))) - kFlatEps;
-  for (int r0 = lo + warp * kCh; r0 <= hi; r0 += kWarps * kCh) {
+  constexpr bool kShare = sizeof(C) == 8;
+  const bool up = a > C(0);
+  for (int r0 = lo + (kShare ? warp * kCh : 0); r0 <= hi; r0 += (kShare ? kWarps : 1) * kCh) {
     const int n = min(kCh, hi - r0 + 1);
     int ylo = 0;
     if constexpr (!ROWS) {
@@ -117,6 +124,7 @@ __device__ __forceinline__ void flat_walk(const Geo<C>& g, const SI* vz, int k, 
       C el = C(1);
       if constexpr (ATT) el = ROWS ? g.ey[(size_t)k * g.ny + line] : g.ex[(size_t)k * g.nx + line];
       const SI* vl = vz + (size_t)line * g.nx * nz;
+      C va[2], wa[2], wb[2];  // value and both weights of the two candidates
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         const int i = i0 + m;
@@ -153,15 +161,37 @@ __device__ __forceinline__ void flat_walk(const Geo<C>& g, const SI* vz, int k, 
           if (line < mine.x || line > mine.y) w0 = C(0);
           if (line < above.x || line > above.y) w = C(0);
         }
-        own = fma(w0, v, own);
-        next = fma(w, v, next);
+        va[m] = v;
+        wa[m] = w0;
+        wb[m] = w;
+      }
+      if constexpr (kShare) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          own = fma(wa[m], va[m], own);
+          next = fma(wb[m], va[m], next);
+        }
+      } else {
+        C vp[2], wp[2];  // those of the bin below, which reach this bin with w
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          vp[m] = __shfl_up_sync(0xffffffffu, va[m], 1);
+          wp[m] = __shfl_up_sync(0xffffffffu, wb[m], 1);
+        }
+        if (up) {  // u grows with the index: the bin below comes first
+          own = fma(wp[1], vp[1], fma(wp[0], vp[0], own));
+          own = fma(wa[1], va[1], fma(wa[0], va[0], own));
+        } else {
+          own = fma(wa[1], va[1], fma(wa[0], va[0], own));
+          own = fma(wp[1], vp[1], fma(wp[0], vp[0], own));
+        }
       }
     }
   }
 }
 
 template <typename SI, typename S, typename C, int MODE, typename O>
-__global__ void __launch_bounds__(kThreads, sizeof(C) == 8 ? 4 : 5)
+__global__ void __launch_bounds__(kThreads, 4)
 k_project_flat(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __restrict__ out,
                const uint8_t* __restrict__ act_col, const int2* __restrict__ rspan, bool wide) {
   if (MODE != kFpStore && b.st->done) return;
@@ -173,13 +203,15 @@ k_project_flat(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O
   StepScalars<C> sc{};
   if (MODE == kFpPrimal || MODE == kFpPrimalCheck) sc = read_scalars<C>(b.st);
   __shared__ C stage[kWarps][flat_rows<C>()][flat_chunk<C>() + 1];
-  __shared__ C psum[kWarps][32];
+  __shared__ C psum[sizeof(C) == 8 ? kWarps : 1][32];
   extern __shared__ __align__(16) unsigned long long kz_block[];
   if constexpr (MODE == kFpCertZ) {
     for (int z = threadIdx.x; z < g.nz; z += blockDim.x) kz_block[z] = 0ull;
     __syncthreads();
   }
-  for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+  constexpr bool kShare = sizeof(C) == 8;
+  for (long long t = kShare ? blockIdx.x : blockIdx.x * kWarps + warp; t < ntiles;
+       t += (kShare ? 1 : kWarps) * gridDim.x) {
     const int k = int(t % g.na);
     const long long t1 = t / g.na;
     const int z = int(t1 % g.nz);
@@ -222,14 +254,17 @@ k_project_flat(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O
       }
 #undef SIPO_FLAT
     }
-    next = __shfl_up_sync(0xffffffffu, next, 1);  // what bin j - 1's voxels give to bin j
-    __syncthreads();  // the previous tile's sums are read
-    psum[warp][lane] = own + next;
-    __syncthreads();
-    if (warp == 0 && live) {
-      C tot[1] = {psum[0][lane]};
+    C tot[1] = {own};
+    if constexpr (kShare) {
+      next = __shfl_up_sync(0xffffffffu, next, 1);  // what bin j - 1's voxels give to bin j
+      __syncthreads();  // the previous tile's sums are read
+      psum[warp][lane] = own + next;
+      __syncthreads();
+      tot[0] = psum[0][lane];
 #pragma unroll
       for (int w = 1; w < kWarps; ++w) tot[0] += psum[w][lane];
+    }
+    if ((!kShare || warp == 0) && live) {
       tot[0] *= esj;
       ZSpan<ZForm<1, 1, false>> zs;
       zs.z0 = z;
@@ -237,10 +272,10 @@ k_project_flat(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O
                                                    kz_block);
     }
   }
-  fp_reduce<MODE, 1>(g, b, red, kz_block, blockIdx.x < ntiles);
+  fp_reduce<MODE, kShare ? 1 : kWarps>(g, b, red, kz_block, blockIdx.x * (kShare ? 1LL : kWarps) < ntiles);
 }
 
-// Views k = first, first + kWarps, ... of one voxel.  Z1: one z value; ES: vial
+// Views k = first, first + kWarps, ... (double precision) or all views of one voxel.  Z1: one z value; ES: vial
 // factors (and ATT: attenuation).
 template <bool ES, bool ATT, bool Z1, typename SI, typename C>
 __device__ __forceinline__ C flat_gather(const Geo<C>& g, const SI* sz, int first, C xf, C yf, int ix, int iy,
@@ -248,18 +283,19 @@ __device__ __forceinline__ C flat_gather(const Geo<C>& g, const SI* sz, int firs
   const int nz = Z1 ? 1 : g.nz;
   C acc = C(0);
   const SI* row = sz + (size_t)first * g.nd * nz;
-  const size_t step = (size_t)kWarps * g.nd * nz;
+  constexpr int kStep = sizeof(C) == 8 ? kWarps : 1;
+  const size_t step = (size_t)kStep * g.nd * nz;
   const int lane = threadIdx.x & 31;
   C shared_inner = C(0);
   int left = 0;  // views whose inner part the lanes still hold
 #pragma unroll 4
-  for (int k = first; k < g.na; k += kWarps, row += step) {
+  for (int k = first; k < g.na; k += kStep, row += step) {
     C inner;
     if constexpr (sizeof(C) == 8) {
       // the row's part of u, one view per lane: FP64 arithmetic is the scarce
       // resource (2 lanes a clock and SM), shuffles are not
       if (left == 0) {
-        const int kl = min(k + lane * kWarps, g.na - 1);
+        const int kl = min(k + lane * kStep, g.na - 1);
         shared_inner = geo_inner(yf, g.cs[2 * kl + 1], g.off);
         left = 32;
       }
@@ -305,8 +341,11 @@ k_backproject_flat(const Geo<C> g, const SI* __restrict__ sino, const Bufs<S, C>
   double red[NR > 0 ? NR : 1] = {};
   StepScalars<C> sc{};
   if (MODE != kBpStore) sc = read_scalars<C>(b.st);
-  __shared__ C psum[kWarps][32];
-  for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+  constexpr bool kShare = sizeof(C) == 8;
+  __shared__ C psum[kShare ? kWarps : 1][32];
+  const int first = kShare ? warp : 0;
+  for (long long t = kShare ? blockIdx.x : blockIdx.x * kWarps + warp; t < ntiles;
+       t += (kShare ? 1 : kWarps) * gridDim.x) {
     const int z = int(t % g.nz);
     const long long t1 = t / g.nz;
     const int ix = int(t1 % ntx) * 32 + lane;
@@ -315,27 +354,30 @@ k_backproject_flat(const Geo<C> g, const SI* __restrict__ sino, const Bufs<S, C>
     const bool in = ix < g.nx && ix >= sp.x && ix <= sp.y && (need == nullptr || need[(size_t)iy * g.nx + ix]);
     const unsigned any = __ballot_sync(0xffffffffu, in);
     C acc = C(0);
-    if (any != 0u) {  // the same for every warp of the block
+    if (any != 0u) {  // (the same for every warp that shares the tile)
       const C xf = C(ix) - g.cx, yf = C(iy) - g.cy;
       const SI* sz = sino + z;
       const int cx = min(ix, g.nx - 1);
       if (g.nz != 1) {
-        acc = g.ex ? flat_gather<true, true, false>(g, sz, warp, xf, yf, cx, iy, in)
-                   : (g.es ? flat_gather<true, false, false>(g, sz, warp, xf, yf, cx, iy, in)
-                           : flat_gather<false, false, false>(g, sz, warp, xf, yf, cx, iy, in));
+        acc = g.ex ? flat_gather<true, true, false>(g, sz, first, xf, yf, cx, iy, in)
+                   : (g.es ? flat_gather<true, false, false>(g, sz, first, xf, yf, cx, iy, in)
+                           : flat_gather<false, false, false>(g, sz, first, xf, yf, cx, iy, in));
       } else {
-        acc = g.ex ? flat_gather<true, true, true>(g, sz, warp, xf, yf, cx, iy, in)
-                   : (g.es ? flat_gather<true, false, true>(g, sz, warp, xf, yf, cx, iy, in)
-                           : flat_gather<false, false, true>(g, sz, warp, xf, yf, cx, iy, in));
+        acc = g.ex ? flat_gather<true, true, true>(g, sz, first, xf, yf, cx, iy, in)
+                   : (g.es ? flat_gather<true, false, true>(g, sz, first, xf, yf, cx, iy, in)
+                           : flat_gather<false, false, true>(g, sz, first, xf, yf, cx, iy, in));
       }
     }
-    __syncthreads();
-    psum[warp][lane] = acc;
-    __syncthreads();
-    if (warp == 0 && ix < g.nx) {
-      C tot[1] = {psum[0][lane]};
+    C tot[1] = {acc};
+    if constexpr (kShare) {
+      __syncthreads();
+      psum[warp][lane] = acc;
+      __syncthreads();
+      tot[0] = psum[0][lane];
 #pragma unroll
       for (int w = 1; w < kWarps; ++w) tot[0] += psum[w][lane];
+    }
+    if ((!kShare || warp == 0) && ix < g.nx) {
       const size_t base = ((size_t)iy * g.nx + ix) * g.nz + z;
       if constexpr (MODE == kBpStore) {
         if (need == nullptr || in) store_z<O, C, 1>(out + base, tot);
@@ -344,7 +386,7 @@ k_backproject_flat(const Geo<C> g, const SI* __restrict__ sino, const Bufs<S, C>
       }
     }
   }
-  if constexpr (MODE == kBpDual) block_reduce_store<2, 0u, 1>(red, b.part, kSlSBand, blockIdx.x < ntiles);
+  if constexpr (MODE == kBpDual) block_reduce_store<2, 0u, kShare ? 1 : kWarps>(red, b.part, kSlSBand, blockIdx.x * (kShare ? 1LL : kWarps) < ntiles);
 }
 
 }  // namespace sipo

@@ -27,8 +27,15 @@ void launch_ray_spans(const Geo<C>& g, const uint8_t* need, int2* out, cudaStrea
 
 // tile: entry of the backprojector tile table.  FP64: 0 = 8 columns per warp, 2
 // blocks/SM; 1 = 4 columns, 2 blocks/SM; 2-6 = 4 columns, 3 blocks/SM.  Single
-// precision: the row-pattern kernel at 2 (0, 1, 3) or 3 (2, 4, 5, 6) blocks/SM.
+// precision: the row-pattern kernel at 2 (0, 1, 3) or 3 (2, 4) blocks/SM; 5, 6 =
+// its form with rows staged by tensor-memory copies where bp_staged allows it,
+// else as 4.
 constexpr int kBpTiles = 7;
+
+// Reads and clears the fault flag of the staged backprojector (bit 0: a bounded
+// wait on a copy gave up; bit 1: rows outside a box; the launch's sums are not
+// valid).  Synchronous: call outside stream capture.
+unsigned int bp_fault_take();
 
 // Runs the bounded mbarrier wait (sipo_wait.cuh) on its own: one
 // block of `threads` threads waits `budget` cycles on a barrier that receives
@@ -53,6 +60,9 @@ void launch_backproject(const Geo<C>& g, const SI* sino, const Bufs<S, C>& b, O*
 template <typename C> inline bool fp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 5 : 8); }
 template <typename C> inline bool bp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 9 : 12); }
 
+// Whether the staged backprojector covers this z extent.
+inline bool bp_staged(int nz) { return nz % 4 == 0; }
+
 // Group size G of the z layout (elements of C in 16 bytes).
 template <typename C> constexpr int z_group() { return 16 / int(sizeof(C)); }
 
@@ -73,9 +83,10 @@ inline int z_group_for(int nz, const A* a, const B* b) {
 // the 16-, 8- or 4-byte loads of a tap plus its fixed part.  E.g. 160^2 x 160,
 // projector: {2, 3} 0.098 ms, {4, 2} 0.113, {4, 1} 0.152.  Double precision
 // keeps two forms of pairs, and single values up to nz = 32, where pairs leave
-// half of the lanes idle (200^2 x 16: 2.70 ms, single 1.81).
+// half of the lanes idle (200^2 x 16: 2.70 ms, single 1.81).  widest: only groups
+// of gmax values (the solver's sums are formed group by group).
 template <typename C, typename F>
-inline void with_z_form(int nz, int gmax, F&& f) {
+inline void with_z_form(int nz, int gmax, F&& f, bool widest = false) {
   if constexpr (sizeof(C) == 8) {
     if (gmax >= 2 && nz % 128 == 0) f(ZForm<2, 2, false>{});
     else if (gmax >= 2 && nz > 32) f(ZForm<2, 1, true>{});
@@ -90,7 +101,7 @@ inline void with_z_form(int nz, int gmax, F&& f) {
     for (int i = 0; i < 10; ++i) {
       const int T = 32 * forms[i].G * forms[i].NG;
       const double cost = ((nz + T - 1) / T) * forms[i].time;
-      if (forms[i].G <= gmax && cost < least) { least = cost; best = i; }
+      if ((widest ? forms[i].G == gmax : forms[i].G <= gmax) && cost < least) { least = cost; best = i; }
     }
     switch (best) {
       case 0: return f(ZForm<4, 2, true>{});

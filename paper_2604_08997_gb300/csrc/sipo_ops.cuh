@@ -317,7 +317,7 @@ k_project(const Geo<C> g, const SI* __restrict__ vol, const Bufs<S, C> b, O* __r
   if (MODE != kFpStore && b.st->done) return;
   constexpr int ZL = Z::ZL;
   constexpr int NR = fp_reductions(MODE);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int warp = threadIdx.x >> 5;
   const int nzc = (g.nz + Z::T - 1) / Z::T;
   const int bw = kWarps / aw;
   const int njb = (g.nd + bw - 1) / bw, nka = (g.na + aw - 1) / aw;
@@ -620,13 +620,14 @@ constexpr int kBp2Generic = 0xff;
 constexpr int kBp2Skip = 0xfe;
 constexpr int kBp2NV = 4;
 
-// Block tiles of k_backproject2: 8 >> split rows of 4 voxels, the views of a row
-// shared by 1 << split warps.  list: the tiles that hold a needed column, as
-// tile row * tiles per row + tile column (nullptr: every tile, n unused).
+// Block tiles of the single-precision backprojector: `rows` rows of 4 voxels, the
+// views of a row shared by 1 << split warps (rows << split <= 8; the
+// order of the sums follows the split, so only the plain operator splits).
+// list: the tiles that hold a needed column, as tile row * tiles per row + tile
+// column (nullptr: every tile, n unused).
 struct BpTiles {
   const int* list;
-  int n;
-  int split;
+  int n, rows, split;
 };
 
 __host__ __device__ constexpr int bp2_off(int pat, int v) { return (pat >> (2 * v)) & 3; }
@@ -770,7 +771,16 @@ __device__ __forceinline__ void bp2_angle(const SI* srow, size_t stride, int nd,
   }
 }
 
-// need, modes and epilogues as in k_backproject.  Each warp sums its share of the
+// Shared memory of one warp: the view table, then the accumulators
+// [voxel][group][lane][G].
+template <typename Z>
+constexpr size_t bp2_warp_bytes() {
+  const size_t table = sizeof(Bp2Ent) * kBp2Chunk, stage = size_t(kBp2NV) * Z::ZL * 32 * sizeof(float);
+  return table > stage ? table : stage;
+}
+
+// Blocks of tiles.rows << tiles.split warps.  need, modes and epilogues as in
+// k_backproject.  Each warp sums its share of the
 // views (a contiguous range, increasing); the shares of a voxel are added in
 // order and finished from shared memory, the groups of a row dealt out to its
 // warps.
@@ -783,19 +793,17 @@ k_backproject2(const Geo<float> g, const SI* __restrict__ sino, const Bufs<S, fl
   if (MODE != kBpStore && b.st->done) return;
   constexpr int NR = MODE == kBpDual ? 2 : 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nsplit = 1 << tiles.split, nrow = kWarps >> tiles.split;
+  const int nsplit = 1 << tiles.split, nrow = tiles.rows;
   const int ntx = (g.nx + NV - 1) / NV, nty = (g.ny + nrow - 1) / nrow;
   const int nzc = (g.nz + Z::T - 1) / Z::T;
   const long long ntiles = (tiles.list ? (long long)tiles.n : (long long)ntx * nty) * nzc;
   double red[NR > 0 ? NR : 1] = {};
   StepScalars<C> sc{};
   if (MODE != kBpStore) sc = read_scalars<C>(b.st);
-  // per warp: the view table, then the accumulators [voxel][group][lane][G]
-  constexpr size_t kTableBytes = sizeof(Bp2Ent) * kBp2Chunk;
-  constexpr size_t kStageBytes = size_t(NV) * Z::ZL * 32 * sizeof(C);
-  constexpr size_t kWarpBytes = kTableBytes > kStageBytes ? kTableBytes : kStageBytes;
-  __shared__ __align__(16) unsigned char smem_warp[kWarps][kWarpBytes];
-  Bp2Ent* tb = reinterpret_cast<Bp2Ent*>(smem_warp[warp]);
+  constexpr size_t kWarpBytes = bp2_warp_bytes<Z>();
+  extern __shared__ __align__(16) unsigned char smem_bp[];
+  unsigned char* smem_warp = smem_bp + warp * kWarpBytes;
+  Bp2Ent* tb = reinterpret_cast<Bp2Ent*>(smem_warp);
   const int ag = warp & (nsplit - 1);
   const int k_lo = int((long long)g.na * ag / nsplit), k_hi = int((long long)g.na * (ag + 1) / nsplit);
   const size_t stride = g.nz;
@@ -847,7 +855,7 @@ k_backproject2(const Geo<float> g, const SI* __restrict__ sino, const Bufs<S, fl
       }
       continue;
     }
-    C* stage = reinterpret_cast<C*>(smem_warp[warp]);
+    C* stage = reinterpret_cast<C*>(smem_warp);
 #pragma unroll
     for (int v = 0; v < NV; ++v)
 #pragma unroll
@@ -858,7 +866,7 @@ k_backproject2(const Geo<float> g, const SI* __restrict__ sino, const Bufs<S, fl
     else __syncwarp();
     if (iy < g.ny) {
       // the epilogue runs group by group to keep its live range short
-      const C* first = reinterpret_cast<const C*>(smem_warp[warp - ag]);
+      const C* first = reinterpret_cast<const C*>(smem_warp - ag * kWarpBytes);
 #pragma unroll 1
       for (int u = ag; u < NV * NG; u += nsplit) {
         const int v = u / NG, q = u % NG;
@@ -881,7 +889,7 @@ k_backproject2(const Geo<float> g, const SI* __restrict__ sino, const Bufs<S, fl
     if (nsplit > 1) __syncthreads();
     else __syncwarp();
   }
-  if constexpr (MODE == kBpDual) block_reduce_store<2>(red, b.part, kSlSBand, blockIdx.x < ntiles);
+  if constexpr (MODE == kBpDual) block_reduce_store<2>(red, b.part, kSlSBand, blockIdx.x < ntiles, int(blockDim.x) / 32);
 }
 
 // ----------------------------------------------------------- ray row spans

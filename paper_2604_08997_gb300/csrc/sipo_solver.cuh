@@ -271,6 +271,14 @@ __device__ __forceinline__ void dual_update(const Bufs<S, C>& b, const StepScala
       if ((kCheckMaxMask >> j) & 1u) red[j] = fmax(red[j], double(acc[j]));
       else red[j] += double(acc[j]);
     }
+  } else if constexpr (ZL == 2 && sizeof(C) == 4) {
+    // pairs come from columns that were summed value by value (nz not a multiple
+    // of 4): the same FP64 terms
+#pragma unroll
+    for (int i = 0; i < ZL; ++i) {
+      if (lab[i] == kBand) red[0] += double(o_lu[i]);
+      else if (lab[i] == kGel) red[1] += double(ft[i] * o_lu[i]);
+    }
   } else {
     red[0] += double(acc[0]);
     red[1] += double(acc[1]);
