@@ -59,7 +59,7 @@ def sm_max_mhz(peaks: dict) -> float:
 # aside) still hash to the value they had at the capture; after any change to
 # the code it is null until re-captured.
 KERNEL_SOURCES = ["sipo_device.cuh", "sipo_solver.cuh", "sipo_ops.cuh", "sipo_launch.h",
-                  "sipo_project.cu", "sipo_backproject.cu", "sipo_bp_tma.cuh"]
+                  "sipo_project.cu", "sipo_backproject.cu", "sipo_bp_tma.cuh", "sipo_pair.cuh", "sipo_wait.cuh"]
 TRAFFIC = {("csg256", "f32"): {"sources_sha256_16": "b793cafb01817e69",
                                "project": 278965120, "backproject": 228099328}}
 

@@ -1550,9 +1550,12 @@ struct Solver final : SolverBase {
     if (!tvol) tvol = dalloc<C>(V);
     std::vector<double> hp(kRedBlocks);
     double* pg = dalloc_part();
-    // b = P_mu^T sino, recomputed (not stored by the forward pass)
+    // b = P_mu^T sino, recomputed (not stored by the forward pass), in the
+    // unsplit order of views: the inner products below cancel, and a change of
+    // order shows in them
+    const BpTiles whole{nullptr, 0, bpt.rows, 0};
     launch_backproject<C, C, C, kBpStore, C>(geo(), static_cast<const C*>(sino), Bufs<C, C>{}, tvol, nullptr,
-                                             s, bpt_all, bp_nv);
+                                             s, whole, bp_nv);
     count(1);
     for (int a = 0; a < 3; ++a) {
       grad[a] = 0.0;

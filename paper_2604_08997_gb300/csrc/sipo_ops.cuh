@@ -85,7 +85,7 @@ __device__ __forceinline__ C tap_weight(C u, C jf, C jm) {
 // Column flags packed as bits for the projector's candidate test.  rows: for
 // each y, bit (x + kNbPad) of word array [y][words] says whether column (y, x)
 // may hold a non-zero input; cols: the same indexed [x][words] by y.  The pad
-// of kNbPad zero bits on both ends lets the three-candidate window be read
+// of kNbPad zero bits on both ends lets a window of up to eight candidates be read
 // without bounds checks (the walk is clipped to spans within the grid).
 constexpr int kNbPad = 32;
 struct NeedBits {
@@ -93,13 +93,14 @@ struct NeedBits {
   const uint32_t* cols;
   int wr, wc;            // words per row / per column
   bool spread;           // flags dilated by a PSF (may lie outside the vial)
+  template <unsigned MASK = 7u>
   __device__ __forceinline__ unsigned window(const uint32_t* base, int line, int start) const {
     const int w = base == rows ? wr : wc;
     int b = start + kNbPad;
-    b = b < 0 ? 0 : (b > 32 * w - 35 ? 32 * w - 35 : b);
+    b = b < 0 ? 0 : (b > 32 * w - 40 ? 32 * w - 40 : b);
     const uint32_t* p = base + (size_t)line * w + (b >> 5);
     const unsigned long long pair = (unsigned long long)__ldg(p) | ((unsigned long long)__ldg(p + 1) << 32);
-    return unsigned(pair >> (b & 31)) & 7u;
+    return unsigned(pair >> (b & 31)) & MASK;
   }
 };
 

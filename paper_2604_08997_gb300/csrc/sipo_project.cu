@@ -3,6 +3,7 @@
 #include "sipo_launch.h"
 #include "sipo_flat.cuh"
 #include "sipo_ops.cuh"
+#include "sipo_pair.cuh"
 
 #include <algorithm>
 
@@ -59,13 +60,20 @@ void launch_project(const Geo<C>& g, const SI* vol, const Bufs<S, C>& b, O* out,
   }
   with_z_form<C>(g.nz, z_group_for<C>(g.nz, vol, out), [&](auto form) {
     using Z = decltype(form);
-    // Views per tile: 4 where every block has several tiles to even out, else 1.
-    // 256^3 x 360 (9.5 tiles a block), solver step: 0.420 ms with 1, 0.394 with 2,
-    // 0.360 with 4, 0.364 with 8 (another target: 0.704, 0.605, 0.616, 0.655);
-    // 96^3 x 391 (4 tiles a block): 0.067 ms with 1, 0.072 with 4.
-    const long long tiles = (long long)g.na * ((g.nd + kWarps - 1) / kWarps) * ((g.nz + Z::T - 1) / Z::T);
-    const int aw = tiles >= 8LL * kRedBlocks ? 4 : 1;
-    k_project<SI, S, C, Z, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan, aw);
+    if constexpr (sizeof(C) == 4 && (MODE == kFpPrimal || MODE == kFpStore)) {
+      // two bins a warp, the same sums; the modes of the check step keep one
+      // (they run once a period).  4 views a tile: 0.344 / 0.560 ms on two targets at
+      // 256^3 x 360, 8 views 0.321 / 0.587; 96^3 x 391 0.0529, 0.0552.
+      k_project_pair<SI, S, Z, MODE, O><<<kRedBlocks, kThreads, 0, stream>>>(g, vol, b, out, act_col, nb, rspan, 4);
+    } else {
+      // Views per tile: 4 where every block has several tiles to even out, else 1.
+      // 256^3 x 360 (9.5 tiles a block): 0.420 ms with 1, 0.394 with 2, 0.360 with 4,
+      // 0.364 with 8 (another target: 0.704, 0.605, 0.616, 0.655); 96^3 x 391 (4
+      // tiles a block): 0.067 ms with 1, 0.072 with 4.
+      const long long tiles = (long long)g.na * ((g.nd + kWarps - 1) / kWarps) * ((g.nz + Z::T - 1) / Z::T);
+      const int aw = tiles >= 8LL * kRedBlocks ? 4 : 1;
+      k_project<SI, S, C, Z, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan, aw);
+    }
   });
 }
 
