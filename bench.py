@@ -60,8 +60,8 @@ def sm_max_mhz(peaks: dict) -> float:
 # the code it is null until re-captured.
 KERNEL_SOURCES = ["sipo_device.cuh", "sipo_solver.cuh", "sipo_ops.cuh", "sipo_launch.h",
                   "sipo_project.cu", "sipo_backproject.cu", "sipo_bp_tma.cuh", "sipo_pair.cuh", "sipo_wait.cuh"]
-TRAFFIC = {("csg256", "f32"): {"sources_sha256_16": "b793cafb01817e69",
-                               "project": 278965120, "backproject": 228099328}}
+TRAFFIC = {("csg256", "f32"): {"sources_sha256_16": "21fd41330c5d655d",
+                               "project": 290100352, "backproject": 218246016}}
 
 
 def _code_only(text: str) -> str:
@@ -512,9 +512,8 @@ def run_gpu(args, dist, rank, world, device):
     fp_ms = phases["project_primal"]
     tr_bp = captured_traffic(args.workload, args.storage, "backproject")
     tr_fp = captured_traffic(args.workload, args.storage, "project")
-    bp_name = {0: "k_backproject", 1: "k_backproject", 2: "k_backproject", 3: "k_backproject2",
-               4: "k_backproject2"}.get(res["tile_cfg"], "k_backproject3")
-    fp_name = "k_project"
+    bp_name = "k_backproject_tma" if res["tile_cfg"] >= 5 else "k_backproject2"
+    fp_name = "k_project" if args.storage == "f64" else "k_project_pair"
     if bp_ms >= fp_ms:
         dom, dom_ms, taps, traffic = f"{bp_name} (fused dual update)", bp_ms, bp_taps, tr_bp
     else:
