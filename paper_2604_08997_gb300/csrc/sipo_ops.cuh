@@ -899,53 +899,46 @@ k_backproject2(const Geo<float> g, const SI* __restrict__ sino, const Bufs<S, fl
 // tests the window of k_project widened by one candidate on each side, so a
 // one-off difference in how the compiler rounds the window start cannot drop
 // a row: restricting the walk to the span skips only rows whose taps are all
-// zero.  Empty spans are (1, 0).
+// zero.  Empty spans are (1, 0).  A warp takes a ray, its lanes 32 lines at a time
+// (one thread a ray took 0.87 ms of the creation of a 512 x 512, 360-view slice).
 template <typename C>
 __global__ void __launch_bounds__(kThreads)
 k_ray_spans(const Geo<C> g, const uint8_t* __restrict__ need, int2* __restrict__ out) {
   const long long n = (long long)g.na * g.nd;
-  for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n;
-       r += (long long)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  for (long long r = blockIdx.x * (long long)kWarps + (threadIdx.x >> 5); r < n;
+       r += (long long)gridDim.x * kWarps) {
     const int k = int(r / g.nd), j = int(r % g.nd);
     const C c = g.cs[2 * k], s = g.cs[2 * k + 1];
     const C jf = C(j);
-    int first = 1, last = 0;
-    if (fabs(c) >= fabs(s)) {
-      const C inv_c = C(1) / c, h = C(1) / fabs(c) + C(kCandEps);
-      for (int iy = 0; iy < g.ny; ++iy) {
-        const int2 sp = g.xspan[iy];
-        if (sp.x > sp.y) continue;
-        const C inner = geo_inner(C(iy) - g.cy, s, g.off);
-        const int ix0 = ceil_int((jf - inner) * inv_c + g.cx - h);
-        bool hit = false;
-        for (int m = -1; m < 4; ++m) {
-          const int ix = ix0 + m;
-          if (ix >= sp.x && ix <= sp.y && need[(size_t)iy * g.nx + ix]) hit = true;
-        }
-        if (hit) {
-          if (first > last) first = iy;
-          last = iy;
-        }
+    const bool rows = fabs(c) >= fabs(s);
+    const C a = rows ? c : s;
+    const C inv_a = C(1) / a, h = C(1) / fabs(a) + C(kCandEps);
+    int first = 0x7fffffff, last = -1;
+    for (int line = lane; line < (rows ? g.ny : g.nx); line += 32) {
+      const int2 sp = rows ? g.xspan[line] : g.yspan[line];
+      if (sp.x > sp.y) continue;
+      int i0;
+      if (rows) {
+        const C inner = geo_inner(C(line) - g.cy, s, g.off);
+        i0 = ceil_int((jf - inner) * inv_a + g.cx - h);
+      } else {
+        const C xf = C(line) - g.cx;
+        i0 = ceil_int((jf - g.off - xf * c) * inv_a + g.cy - h);
       }
-    } else {
-      const C inv_s = C(1) / s, h = C(1) / fabs(s) + C(kCandEps);
-      for (int ix = 0; ix < g.nx; ++ix) {
-        const int2 sp = g.yspan[ix];
-        if (sp.x > sp.y) continue;
-        const C xf = C(ix) - g.cx;
-        const int iy0 = ceil_int((jf - g.off - xf * c) * inv_s + g.cy - h);
-        bool hit = false;
-        for (int m = -1; m < 4; ++m) {
-          const int iy = iy0 + m;
-          if (iy >= sp.x && iy <= sp.y && need[(size_t)iy * g.nx + ix]) hit = true;
-        }
-        if (hit) {
-          if (first > last) first = ix;
-          last = ix;
-        }
+      bool hit = false;
+      for (int m = -1; m < 4; ++m) {
+        const int i = i0 + m;
+        if (i >= sp.x && i <= sp.y && need[rows ? (size_t)line * g.nx + i : (size_t)i * g.nx + line]) hit = true;
+      }
+      if (hit) {
+        first = min(first, line);
+        last = line;
       }
     }
-    out[r] = make_int2(first, last);
+    first = __reduce_min_sync(0xffffffffu, first);
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0) out[r] = last < 0 ? make_int2(1, 0) : make_int2(first, last);
   }
 }
 

@@ -88,7 +88,7 @@ void launch_need_bits(const uint8_t* need, uint32_t* rows, uint32_t* cols, int n
 template <typename C>
 void launch_ray_spans(const Geo<C>& g, const uint8_t* need, int2* out, cudaStream_t stream) {
   const long long n = (long long)g.na * g.nd;
-  const int grid = int(std::min<long long>((n + kThreads - 1) / kThreads, (long long)device_sms() * 16));
+  const int grid = int(std::min<long long>((n + kWarps - 1) / kWarps, (long long)device_sms() * 16));
   k_ray_spans<C><<<grid, kThreads, 0, stream>>>(g, need, out);
 }
 template void launch_ray_spans<float>(const Geo<float>&, const uint8_t*, int2*, cudaStream_t);
