@@ -60,8 +60,8 @@ def sm_max_mhz(peaks: dict) -> float:
 # the code it is null until re-captured.
 KERNEL_SOURCES = ["sipo_device.cuh", "sipo_solver.cuh", "sipo_ops.cuh", "sipo_launch.h",
                   "sipo_project.cu", "sipo_backproject.cu", "sipo_bp_tma.cuh", "sipo_pair.cuh", "sipo_wait.cuh"]
-TRAFFIC = {("csg256", "f32"): {"sources_sha256_16": "21fd41330c5d655d",
-                               "project": 290100352, "backproject": 218246016}}
+TRAFFIC = {("csg256", "f32"): {"sources_sha256_16": "9ebeb4d949b906e3",
+                               "project": 289981696, "backproject": 218191104}}
 
 
 def _code_only(text: str) -> str:
