@@ -77,16 +77,17 @@ __device__ __forceinline__ int fp2_line_taps(const Geo<float>& g, const NeedBits
     const bool ok = (okm >> m) & 1u;
     ta = ok && in_a ? ta : 0.0f;
     tb = ok && in_b ? tb : 0.0f;
-    const bool tap = ta != 0.0f || tb != 0.0f;
     const int ix = ROWS ? i0 + m : line, iy = ROWS ? line : i0 + m;
-    if (g.ex && tap) {
+    if (g.ex && (ta != 0.0f || tb != 0.0f)) {
       const float e = ROWS ? g.ex[(size_t)ray.k * g.nx + ix] * eline : eline * g.ey[(size_t)ray.k * g.ny + iy];
-      ta *= e;
-      tb *= e;
+      ta = ta != 0.0f ? ta * e : 0.0f;  // (e may be infinite: a bin out of reach stays at zero)
+      tb = tb != 0.0f ? tb * e : 0.0f;
     }
     col[m] = iy * g.nx + ix;
     wt[m] = make_float2(ta, tb);
-    nt += tap;
+    // counted by the weights that fp2_walk lists: a strong attenuation may have
+    // brought both to zero, and a place reserved for them would stay unwritten
+    nt += ta != 0.0f || tb != 0.0f;
   }
   return nt;
 }
@@ -123,6 +124,7 @@ __device__ __forceinline__ void fp2_walk(const Geo<float>& g, const SI* vz, cons
         ++pos;
       }
     }
+    SIPO_DCHECK(pos == incl, 0);
     __syncwarp();
 #ifdef SIPO_CHECKED
     for (int q = lane; q < total; q += 32) SIPO_DCHECK((unsigned(tl.col[q]) < unsigned(g.nx * g.ny)), 0);
