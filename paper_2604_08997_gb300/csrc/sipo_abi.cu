@@ -775,6 +775,13 @@ struct Solver final : SolverBase {
   }
 
   // ---------------------------------------------------------------- PSF
+  // Whether groups of four z values of a caller's buffer can be moved in one
+  // access (FP64 moves them one by one).
+  template <typename T>
+  static bool quad_aligned(const T* p) {
+    return sizeof(T) == 8 || reinterpret_cast<uintptr_t>(p) % (4 * sizeof(T)) == 0;
+  }
+
   // in -> out through the three axis passes (taps or, on deriv_axis, their
   // sigma derivative).  tmp_a and tmp_b are C volumes distinct from in/out.
   template <typename TI, typename TO>
@@ -783,10 +790,10 @@ struct Solver final : SolverBase {
     for (int a = 0; a < 3; ++a) tp[a] = (deriv == a) ? dtaps[a] : taps[a];
     // an axis without blur runs the single tap 1 (R = 0): a copy
     if constexpr (sizeof(C) == 4) {
-      // single precision, nz % 4 == 0: x and y in one pass through shared
-      // memory, then z from shared-memory chunks
+      // single precision, nz % 4 == 0, aligned buffers: x and y in one pass
+      // through shared memory, then z from shared-memory chunks
       const size_t smem = conv_xy_smem(R[0], R[1]);
-      if (nz % 4 == 0 && smem <= 227 * 1024 && R[2] <= kZMaxR) {
+      if (nz % 4 == 0 && quad_aligned(in) && quad_aligned(out) && smem <= 227 * 1024 && R[2] <= kZMaxR) {
         const float* tpx = reinterpret_cast<const float*>(tp[0] ? tp[0] : unit_tap());
         const float* tpy = reinterpret_cast<const float*>(tp[1] ? tp[1] : unit_tap());
         const float* tpz = reinterpret_cast<const float*>(tp[2] ? tp[2] : unit_tap());
@@ -810,10 +817,11 @@ struct Solver final : SolverBase {
     count(3);
   }
 
-  // One axis pass: VG = 4 z values per thread when nz % 4 == 0.
+  // One axis pass: VG = 4 z values per thread when nz % 4 == 0 and the buffers
+  // are aligned.
   template <typename TI, typename TO>
   void conv_pass(const TI* in, TO* out, const C* tp, int r, int axis, cudaStream_t s) {
-    const int vg = nz % 4 == 0 ? 4 : 1;
+    const int vg = nz % 4 == 0 && quad_aligned(in) && quad_aligned(out) ? 4 : 1;
     const int nzg = nz / vg;
     long long nb;
     if (axis < 2) {
