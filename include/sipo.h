@@ -246,7 +246,8 @@ int sipo_response_metrics(sipo_ctx *ctx, const sipo_response *M, const float *m_
  * is SIPO_F64), host or device per y_location.  Blocks until done.  Errors:
  * INVALID_ARG, CUDA, TIMEOUT (a bounded device-side wait of the staged
  * backprojector gave up), NUMERIC (a check found NaN or infinite residuals,
- * e.g. from an infinite imported start); the context stays usable. */
+ * e.g. from an infinite imported start; or detector rows outside a staged box,
+ * which the geometry cannot produce); the context stays usable. */
 int sipo_solve(sipo_ctx *ctx, void *y_out, int y_location, sipo_result *res);
 
 /* Warm start, for precision escalation (a reading of the mixed-precision
@@ -389,7 +390,12 @@ int sipo_solve_batched(sipo_ctx **ctxs, int n, void **y_outs, int y_location,
  * one context must not overlap in time on different streams. */
 int sipo_project(sipo_ctx *ctx, const void *vol, void *sino, int dtype, void *stream);
 
-/* A^T sino = K P_mu^T sino (Eq. 3); arguments as sipo_project. */
+/* A^T sino = K P_mu^T sino (Eq. 3); arguments as sipo_project.  The staged
+ * backprojector bounds its device-side waits; a launch whose wait gave up has
+ * not written all of vol and records a fault in the context.  The call has
+ * returned by then: the fault is reported, once, as TIMEOUT by the context's
+ * next sipo_project, sipo_backproject, sipo_psf_grad (which also reports its
+ * own), solve or sipo_check_fault. */
 int sipo_backproject(sipo_ctx *ctx, const void *sino, void *vol, int dtype, void *stream);
 
 /* K vol (deriv_axis < 0) or (dK/dsigma_a) vol for a = deriv_axis in {0:x,
@@ -406,6 +412,18 @@ int sipo_psf_apply(sipo_ctx *ctx, const void *in, void *out, int dtype, int deri
  * vol are device arrays of `dtype`; axes without a PSF get 0. */
 int sipo_psf_grad(sipo_ctx *ctx, const void *sino, const void *vol, int dtype, double *grad,
                   void *stream);
+
+/* Reports the fault that earlier launches of this context have recorded and
+ * clears it: SIPO_OK, TIMEOUT (a bounded device-side wait gave up) or NUMERIC
+ * (detector rows outside a staged box, which the geometry cannot produce).
+ * Does not synchronise: after a synchronisation of the stream of a
+ * sipo_backproject it says whether that call's sums are valid. */
+int sipo_check_fault(sipo_ctx *ctx);
+
+/* Self-test: records a fault in the context as a launch would (bit 0: a wait
+ * that gave up, bit 1: rows outside a box).  Nothing is launched.  Errors:
+ * INVALID_ARG (null, bits outside 1..3). */
+int sipo_post_fault(sipo_ctx *ctx, unsigned int bits);
 
 /* Replaces the PSF sigmas (radii stay frozen); affects later operator calls. */
 int sipo_set_psf_sigma(sipo_ctx *ctx, const double sigma[3]);

@@ -118,6 +118,8 @@ SIGNATURES = {
     "sipo_phase_name": (c_char_p, [c_int]),
     "sipo_tile_count": (c_int, []),
     "sipo_check_flags": (ctypes.c_uint, []),
+    "sipo_check_fault": (c_int, [c_void_p]),
+    "sipo_post_fault": (c_int, [c_void_p, ctypes.c_uint]),
     "sipo_wait_selftest": (c_int, [c_longlong, c_int, c_int, POINTER(ctypes.c_uint)]),
     "sipo_kernel_launch_count": (c_longlong, []),
     "sipo_set_tolerances": (c_int, [c_void_p, POINTER(sipo_tolerances)]),
@@ -517,6 +519,18 @@ def sipo_kernel_launch_count() -> int:
 def sipo_tile_count() -> int:
     """Entries of the backprojector tile table (values of tolerances["tile_cfg"])."""
     return int(load().sipo_tile_count())
+
+
+def sipo_check_fault(ctx: Context):
+    """Raises SipoError if an earlier launch of this context recorded a fault (see
+    include/sipo.h), and clears it.  Does not synchronise."""
+    _check(load().sipo_check_fault(ctx.handle))
+
+
+def sipo_post_fault(ctx: Context, bits: int):
+    """Self-test: records a fault as a launch would (bit 0: a wait that gave up,
+    bit 1: rows outside a staged box)."""
+    _check(load().sipo_post_fault(ctx.handle, int(bits)))
 
 
 def sipo_wait_selftest(budget_cycles: int, arrive: bool, threads: int = 128) -> tuple[int, int]:

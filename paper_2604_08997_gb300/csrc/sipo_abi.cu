@@ -71,6 +71,9 @@ struct SolverBase {
   virtual void psf_apply(const void* in, void* out, int deriv, cudaStream_t s) = 0;
   virtual void psf_grad(const void* sino, const void* vol, double* grad, cudaStream_t s) = 0;
   virtual void set_sigma(const double* sig) = 0;
+  // throws if an earlier launch of this context recorded a fault, and clears it
+  virtual void check_fault() = 0;
+  virtual void post_fault(unsigned int bits) = 0;
   virtual void get_array(int which, void* out, int loc) = 0;
   virtual void profile(int iters, double* ms, int n) = 0;
   virtual int compute_dtype() const = 0;
@@ -160,7 +163,7 @@ struct Solver final : SolverBase {
   int ze = 1;  // elements per thread of the element-wise kernels
   // block tiles of the single-precision backprojector: those with a needed
   // column (solver steps), and all (the plain operator)
-  BpTiles bpt{nullptr, 0, 8, 0}, bpt_all{nullptr, 0, 8, 0};
+  BpTiles bpt{nullptr, 0, 8, 0, nullptr}, bpt_all{nullptr, 0, 8, 0, nullptr};
   int P = 64;
   bool psf = false;
   int bp_nv = 0;     // backprojector tile table entry
@@ -198,6 +201,7 @@ struct Solver final : SolverBase {
   double* trace = nullptr;
   static constexpr int kTraceCap = 4096;
   Scal* h_st = nullptr;  // pinned host mirror
+  volatile unsigned int* h_fault = nullptr;  // fault words of the staged backprojector, mapped
 
   // host constants
   bool ft_is_const = false;
@@ -249,6 +253,14 @@ struct Solver final : SolverBase {
       own_stream = true;
     }
     ck(cudaHostAlloc(reinterpret_cast<void**>(&h_st), sizeof(Scal), cudaHostAllocDefault), "cudaHostAlloc");
+    unsigned int* fault = nullptr;
+    ck(cudaHostAlloc(reinterpret_cast<void**>(&fault), 2 * sizeof(unsigned int), cudaHostAllocMapped),
+       "cudaHostAlloc");
+    fault[0] = fault[1] = 0u;
+    h_fault = fault;
+    unsigned int* mapped = nullptr;
+    ck(cudaHostGetDevicePointer(reinterpret_cast<void**>(&mapped), fault, 0), "fault words");
+    bpt.fault = bpt_all.fault = mapped;
   }
 
   ~Solver() override {
@@ -257,6 +269,7 @@ struct Solver final : SolverBase {
     for (void* p : allocs) cudaFree(p);
     if (tconv) cudaFree(tconv);
     if (h_st) cudaFreeHost(h_st);
+    if (h_fault) cudaFreeHost(const_cast<unsigned int*>(h_fault));
     if (own_stream && stream) cudaStreamDestroy(stream);
   }
 
@@ -277,6 +290,7 @@ struct Solver final : SolverBase {
   }
 
   void init_for_batch() override {
+    check_fault();
     if (!warm_pending) init_state();
     warm_pending = false;
     launches = 0;
@@ -437,7 +451,7 @@ struct Solver final : SolverBase {
     ck(cudaGetLastError(), "Farkas test");
     ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
     ck(cudaStreamSynchronize(stream), "Farkas test");
-    check_bp_fault();
+    check_fault();
     const int cert = h_st->cert;
     if (slice) *slice = cert ? h_st->cert_z : -1;
     init_state();
@@ -517,6 +531,7 @@ struct Solver final : SolverBase {
     *h_st = h;
     ck(cudaMemcpyAsync(st, h_st, sizeof(Scal), cudaMemcpyHostToDevice, stream), "state");
     ck(cudaStreamSynchronize(stream), "state start");
+    check_fault();
     warm_pending = true;
   }
 
@@ -1113,7 +1128,7 @@ struct Solver final : SolverBase {
     k_apply_mask<C><<<gs, kThreads, 0, stream>>>(col, mask, (long long)SN);
     // row abs-sums of A^T over active rays: A^T 1_act = K P^T 1_act, in the
     // solver's order of views
-    const BpTiles whole{nullptr, 0, bpt.rows, 0};
+    const BpTiles whole{nullptr, 0, bpt.rows, 0, bpt.fault};
     if (psf) {
       launch_backproject<C, C, C, kBpStore, C>(g, g0, Bufs<C, C>{}, t1, nullptr, stream, whole);
       psf3<C, C>(t1, row, t2, t3, -1, stream);
@@ -1186,6 +1201,7 @@ struct Solver final : SolverBase {
   }
 
   void begin_solve() override {
+    check_fault();
     if (!warm_pending) init_state();
     warm_pending = false;
     build_graph();
@@ -1433,7 +1449,7 @@ struct Solver final : SolverBase {
   void finish_solve(void* y_out, int loc, sipo_result* res) override {
     ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
     ck(cudaStreamSynchronize(stream), "solve");
-    check_bp_fault();
+    check_fault();
     if (!h_st->done) {
       final_check();
       ck(cudaMemcpyAsync(h_st, st, sizeof(Scal), cudaMemcpyDeviceToHost, stream), "read state");
@@ -1457,6 +1473,7 @@ struct Solver final : SolverBase {
     ck(cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, stream), "metrics");
     if (y_out) copy_out(yp, SN, y_out, loc, conv_tmp(SN));
     ck(cudaStreamSynchronize(stream), "metrics");
+    check_fault();
     double m[8] = {1e300, -1e300, -1e300, 1e300, 0.0, 0.0, 1e300, -1e300};
     for (int b = 0; b < kRedBlocks; ++b) {
       m[0] = std::min(m[0], hp[0 * kRedBlocks + b]);
@@ -1490,13 +1507,19 @@ struct Solver final : SolverBase {
     res->cert_slice = h.status == 1 ? h.cert_z : -1;
   }
 
-  // A bounded wait inside the staged backprojector gave up (bit 0), or a view's
-  // rows did not fit its box (bit 1): the sums of that launch are not valid, so
-  // the solve is an error.
-  void check_bp_fault() {
-    const unsigned int f = bp_fault_take();
-    if (f & 1u) fail(SIPO_ERR_TIMEOUT, "backprojector: a wait on a tensor-memory copy timed out");
-    if (f) fail(SIPO_ERR_NUMERIC, "backprojector: detector rows outside the staged box");
+  // A bounded wait inside the staged backprojector gave up (word 0), or a view's
+  // rows did not fit its box (word 1): the sums of that launch are not valid.
+  // Does not synchronise: sees the launches that have ended.
+  void check_fault() override {
+    const unsigned int wait = h_fault[0], box = h_fault[1];
+    h_fault[0] = h_fault[1] = 0u;
+    if (wait) fail(SIPO_ERR_TIMEOUT, "backprojector: a wait on a tensor-memory copy timed out");
+    if (box) fail(SIPO_ERR_NUMERIC, "backprojector: detector rows outside the staged box");
+  }
+
+  void post_fault(unsigned int bits) override {
+    if (bits & 1u) h_fault[0] = 1u;
+    if (bits & 2u) h_fault[1] = 1u;
   }
 
   // copies n elements of S (converted to C) to out (host or device)
@@ -1561,7 +1584,7 @@ struct Solver final : SolverBase {
     // b = P_mu^T sino, recomputed (not stored by the forward pass), in the
     // unsplit order of views: the inner products below cancel, and a change of
     // order shows in them
-    const BpTiles whole{nullptr, 0, bpt.rows, 0};
+    const BpTiles whole{nullptr, 0, bpt.rows, 0, bpt.fault};
     launch_backproject<C, C, C, kBpStore, C>(geo(), static_cast<const C*>(sino), Bufs<C, C>{}, tvol, nullptr,
                                              s, whole, bp_nv);
     count(1);
@@ -1575,6 +1598,7 @@ struct Solver final : SolverBase {
       ck(cudaStreamSynchronize(s), "psf grad");
       for (int i = 0; i < kRedBlocks; ++i) grad[a] += hp[i];
     }
+    check_fault();
   }
 
   double* gpart = nullptr;
@@ -2058,6 +2082,7 @@ int sipo_project(sipo_ctx* ctx, const void* vol, void* sino, int dtype, void* st
   check_dtype(ctx, dtype);
   if (!vol || !sino) sipo::fail(SIPO_ERR_INVALID_ARG, "null buffer");
   cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : ctx->c.s->strm();
+  ctx->c.s->check_fault();
   ctx->c.s->project(vol, sino, s);
   return SIPO_OK;
   SIPO_CATCH
@@ -2068,6 +2093,7 @@ int sipo_backproject(sipo_ctx* ctx, const void* sino, void* vol, int dtype, void
   check_dtype(ctx, dtype);
   if (!vol || !sino) sipo::fail(SIPO_ERR_INVALID_ARG, "null buffer");
   cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : ctx->c.s->strm();
+  ctx->c.s->check_fault();
   ctx->c.s->backproject(sino, vol, s);
   return SIPO_OK;
   SIPO_CATCH
@@ -2088,7 +2114,24 @@ int sipo_psf_grad(sipo_ctx* ctx, const void* sino, const void* vol, int dtype, d
   check_dtype(ctx, dtype);
   if (!sino || !vol || !grad) sipo::fail(SIPO_ERR_INVALID_ARG, "null buffer");
   cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : ctx->c.s->strm();
+  ctx->c.s->check_fault();
   ctx->c.s->psf_grad(sino, vol, grad, s);
+  return SIPO_OK;
+  SIPO_CATCH
+}
+
+int sipo_check_fault(sipo_ctx* ctx) {
+  SIPO_TRY
+  if (!ctx) sipo::fail(SIPO_ERR_INVALID_ARG, "null argument");
+  ctx->c.s->check_fault();
+  return SIPO_OK;
+  SIPO_CATCH
+}
+
+int sipo_post_fault(sipo_ctx* ctx, unsigned int bits) {
+  SIPO_TRY
+  if (!ctx || bits == 0 || bits > 3) sipo::fail(SIPO_ERR_INVALID_ARG, "null context or bits outside 1..3");
+  ctx->c.s->post_fault(bits);
   return SIPO_OK;
   SIPO_CATCH
 }

@@ -27,16 +27,6 @@ unsigned int check_flags_backproject() {
 }
 
 
-unsigned int bp_fault_take() {
-  unsigned int v = 0;
-  if (cudaMemcpyFromSymbol(&v, g_bp_fault, sizeof(v)) != cudaSuccess) return 0;
-  if (v) {
-    const unsigned int zero = 0;
-    cudaMemcpyToSymbol(g_bp_fault, &zero, sizeof(zero));
-  }
-  return v;
-}
-
 int wait_selftest(long long budget, int arrive, int threads, unsigned int* timed_out) {
   unsigned int* d = nullptr;
   if (cudaMalloc(&d, sizeof(unsigned int)) != cudaSuccess) return -1;

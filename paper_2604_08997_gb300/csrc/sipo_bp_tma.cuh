@@ -20,8 +20,8 @@
 // 0.72 ms (14.6 -> 23 TFLOP/s) where the rows read through L1 took 1.12 ms; solver
 // steps 0.326 ms (0.471 through L1) and, on a larger part, 0.493 ms (0.611).
 //
-// Waits are bounded: one that outlives kWaitCycles sets a fault flag (read by
-// bp_fault_take on the host) and the block's abort flag, on which every wait
+// Waits are bounded: one that outlives kWaitCycles sets the context's fault word
+// (tiles.fault, read by the host) and the block's abort flag, on which every wait
 // ends; the copying warp then waits (bounded) for its copies in flight.
 #pragma once
 
@@ -35,10 +35,6 @@ namespace sipo {
 template <int ROWS> constexpr int bt_bins() { return ROWS == 8 ? 10 : 6; }  // per staged box
 constexpr int kBtViews = 2;     // views per stage
 constexpr int kBtStages = 4;    // stages of the ring
-
-// Fault flag (bit 0: a wait on a copy or on a reader gave up).  Defined here:
-// one translation unit (sipo_backproject.cu) includes this file.
-__device__ unsigned int g_bp_fault = 0;
 
 // One box of the 3-D tensor map (z, bin, view) into shared memory, completing
 // on `bar` (its byte count is announced by mbar_expect_tx).
@@ -71,13 +67,14 @@ struct BtSmem {
 };
 
 // Wait that also ends when the block aborts.
-__device__ __forceinline__ bool bt_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+__device__ __forceinline__ bool bt_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                        volatile unsigned int* fault) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity)) {
     if (*abort_flag) return false;
     if (clock64() - t0 > kWaitCycles) {
-      atomicOr(&g_bp_fault, 1u);
+      fault[0] = 1u;
       *abort_flag = 1;
       return false;
     }
@@ -214,7 +211,7 @@ k_backproject_tma(const Geo<float> g, const __grid_constant__ CUtensorMap tmap, 
           int good = 1;
           if (lane == 0) {
             // the slot's readers of the round before are done
-            if (round > 0) good = bt_wait(empty + slot, (round - 1) & 1u, abort_flag);
+            if (round > 0) good = bt_wait(empty + slot, (round - 1) & 1u, abort_flag, tiles.fault);
             if (good) {
               const int n = min(kBtViews, kn - a);
               unsigned char* dst = smem + slot * SM::kStageBytes;
@@ -277,7 +274,7 @@ k_backproject_tma(const Geo<float> g, const __grid_constant__ CUtensorMap tmap, 
             // (a span wider than the box, which these tiles cannot have, is not read)
             if (o.row < 0 || max(max(e.i0.x, e.i0.y), max(e.i0.z, e.i0.w)) + 1 - b0 >= bt_bins<ROWS>()) {
               o.pat = kBp2Skip;
-              atomicOr(&g_bp_fault, 2u);
+              tiles.fault[1] = 1u;
             }
             tb[lane] = o;
           }
@@ -286,7 +283,7 @@ k_backproject_tma(const Geo<float> g, const __grid_constant__ CUtensorMap tmap, 
             const unsigned slot = seq % kBtStages;
             // the entries do not depend on the copies: read ahead of the wait
             const BtEnt e0 = tb[a], e1 = tb[min(a + 1, kBp2Chunk - 1)];
-            ok = bt_wait(full + slot, (seq / kBtStages) & 1u, abort_flag);
+            ok = bt_wait(full + slot, (seq / kBtStages) & 1u, abort_flag, tiles.fault);
             if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
             if (mask != 0u) {
               const SI* box = reinterpret_cast<const SI*>(smem + slot * SM::kStageBytes) + lane * 4;

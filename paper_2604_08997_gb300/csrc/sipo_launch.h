@@ -32,11 +32,6 @@ void launch_ray_spans(const Geo<C>& g, const uint8_t* need, int2* out, cudaStrea
 // else as 4.
 constexpr int kBpTiles = 7;
 
-// Reads and clears the fault flag of the staged backprojector (bit 0: a bounded
-// wait on a copy gave up; bit 1: rows outside a box; the launch's sums are not
-// valid).  Synchronous: call outside stream capture.
-unsigned int bp_fault_take();
-
 // Runs the bounded mbarrier wait (sipo_wait.cuh) on its own: one
 // block of `threads` threads waits `budget` cycles on a barrier that receives
 // its one arrival only if `arrive`; *timed_out = threads whose wait gave up.

@@ -625,10 +625,13 @@ constexpr int kBp2NV = 4;
 // views of a row shared by 1 << split warps (rows << split <= 8; the
 // order of the sums follows the split, so only the plain operator splits).
 // list: the tiles that hold a needed column, as tile row * tiles per row + tile
-// column (nullptr: every tile, n unused).
+// column (nullptr: every tile, n unused).  fault: the context's fault words in
+// mapped host memory, set to 1 by a staged launch whose sums are not valid
+// ([0]: a bounded wait gave up, [1]: rows outside a box).
 struct BpTiles {
   const int* list;
   int n, rows, split;
+  volatile unsigned int* fault;
 };
 
 __host__ __device__ constexpr int bp2_off(int pat, int v) { return (pat >> (2 * v)) & 3; }
