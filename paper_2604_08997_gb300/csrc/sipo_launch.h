@@ -52,7 +52,11 @@ void launch_backproject(const Geo<C>& g, const SI* sino, const Bufs<S, C>& b, O*
 // projector 274 / 115 at nz = 4, 277 / 246 at 8, 279 / 349 at 12; backprojector
 // 317 / 149 at 8, 317 / 209 at 12, 319 / 411 at 16; double precision, projector
 // 2696 / 1859 at 4, 2696 / 2738 at 6; backprojector 2387 / 1950 at 8, 2480 / 2879 at 12.
-template <typename C> inline bool fp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 5 : 8); }
+// The flat projector's candidate window holds up to sides (and detectors) of kFlatSide.
+constexpr int kFlatSide = 16384;
+template <typename C> inline bool fp_flat(const Geo<C>& g) {
+  return g.nz <= (sizeof(C) == 8 ? 5 : 8) && g.nx <= kFlatSide && g.ny <= kFlatSide && g.nd <= kFlatSide;
+}
 template <typename C> inline bool bp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 9 : 12); }
 
 // Whether the staged backprojector covers this z extent.

@@ -51,7 +51,7 @@ void launch_project(const Geo<C>& g, const SI* vol, const Bufs<S, C>& b, O* out,
                     const int2* rspan) {
   // the slice-mode certificate keeps one 8-byte maximum per z in shared memory
   const size_t dyn = MODE == kFpCertZ ? size_t(g.nz) * sizeof(unsigned long long) : 0;
-  if (fp_flat<C>(g.nz)) {
+  if (fp_flat<C>(g)) {
     // a solver's input vanishes outside its flagged columns; those may lie
     // outside the vial where a PSF spreads them
     const bool wide = nb.rows != nullptr && g.r2i >= 0 && nb.spread;
