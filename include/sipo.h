@@ -387,10 +387,14 @@ int sipo_solve_batched(sipo_ctx **ctxs, int n, void **y_outs, int y_location,
 /* A vol = P_mu K vol (the adjoint of Eq. 3): vol is a device volume, sino a
  * device sinogram, both of `dtype` (SIPO_F32 or SIPO_F64).  Enqueued on
  * `stream`.  With a PSF, uses a context-owned temporary volume, so calls on
- * one context must not overlap in time on different streams. */
+ * one context must not overlap in time on different streams.  Without a PSF an
+ * infinite or NaN voxel makes the bins non-finite that weigh it and leaves every
+ * other bin as it is; K spreads it over its radii first. */
 int sipo_project(sipo_ctx *ctx, const void *vol, void *sino, int dtype, void *stream);
 
-/* A^T sino = K P_mu^T sino (Eq. 3); arguments as sipo_project.  The staged
+/* A^T sino = K P_mu^T sino (Eq. 3); arguments as sipo_project.  An infinite or
+ * NaN bin may also reach neighbouring voxels that weigh it with zero (as
+ * 0 * inf), those outside the vial among them.  The staged
  * backprojector bounds its device-side waits; a launch whose wait gave up has
  * not written all of vol and records a fault in the context.  The call has
  * returned by then: the fault is reported, once, as TIMEOUT by the context's

@@ -5,8 +5,10 @@
 // Here a warp sums two neighbouring bins of one view: a column that reaches either
 // is loaded once (3.4 a line for 4.5 taps), with a weight for each bin, one of
 // them zero for the outer columns.  Taps keep the order of the per-ray walk, and
-// a zero weight leaves a sum unchanged, so the sums are those of k_project bit for
-// bit.  (Four bins a warp, without zero weights through 13 line shapes, moved even
+// a zero weight leaves a sum of finite values unchanged, so the sums are those of
+// k_project bit for bit.  An infinite or NaN voxel would reach the other bin as
+// 0 * inf: the plain operator sums a pair that came out NaN again, one bin at a
+// time.  (Four bins a warp, without zero weights through 13 line shapes, moved even
 // less but was slower: 16 to 24 warps an SM could not cover a line's chain of
 // table, jump, loads and multiply-adds.)
 //
@@ -35,6 +37,7 @@ struct PairList {
 struct PairRay {
   float c, s, inv_a, h;  // h: half the candidate window with its margin
   int k, j;
+  unsigned bins;         // bit 0: bin j is summed, bit 1: bin j + 1
   bool spread;           // per-bin line ranges apply (flags outside the vial)
   int2 ra, rb;           // line ranges of bins j and j + 1
 };
@@ -66,8 +69,8 @@ __device__ __forceinline__ int fp2_line_taps(const Geo<float>& g, const NeedBits
   const float f0 = ROWS ? cf - g.cx : cf - g.cy;
   float eline = 1.0f;
   if (g.ex) eline = ROWS ? g.ey[(size_t)ray.k * g.ny + line] : g.ex[(size_t)ray.k * g.nx + line];
-  const bool in_a = !ray.spread || (line >= ray.ra.x && line <= ray.ra.y);
-  const bool in_b = !ray.spread || (line >= ray.rb.x && line <= ray.rb.y);
+  const bool in_a = (ray.bins & 1u) && (!ray.spread || (line >= ray.ra.x && line <= ray.ra.y));
+  const bool in_b = (ray.bins & 2u) && (!ray.spread || (line >= ray.rb.x && line <= ray.rb.y));
   int nt = 0;
 #pragma unroll
   for (int m = 0; m < kPairVox; ++m) {
@@ -214,28 +217,41 @@ k_project_pair(const Geo<float> g, const SI* __restrict__ vol, const Bufs<S, flo
     const int lo = min(range[0].x, range[1].x), hi = max(range[0].y, range[1].y);
     ZSpan<Z> zs;
     zs.init(g.nz, tz);
-    float acc[2][ZL];
-#pragma unroll
-    for (int i = 0; i < ZL; ++i) acc[0][i] = acc[1][i] = 0.0f;
     const SI* vz = vol + zs.z0;
     PairList& tl = taps[warp];
-    if (rows) {
-      if (j0 >= 2) fp2_walk<true, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
-      else fp2_walk<true, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
-    } else {
-      if (j0 >= 2) fp2_walk<false, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
-      else fp2_walk<false, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
-    }
-    if (Z::kRagged && zs.fresh == 0u) continue;
-    SIPO_DCHECK(zs.z0 + zs.at(Z::NG - 1) + Z::G - 1 < g.nz, 0);
+    // both bins together; a pair that came out NaN again, one after the other
+    for (unsigned bins = 3u; bins != 0u;) {
+      ray.bins = bins;
+      float acc[2][ZL];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (!((live >> q) & 1u)) continue;
-      const size_t at = (size_t)k * g.nd + j0 + q;
-      const float es = g.es ? g.es[at] : 1.0f;
+      for (int i = 0; i < ZL; ++i) acc[0][i] = acc[1][i] = 0.0f;
+      if (rows) {
+        if (j0 >= 2) fp2_walk<true, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+        else fp2_walk<true, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+      } else {
+        if (j0 >= 2) fp2_walk<false, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+        else fp2_walk<false, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+      }
+      if (MODE == kFpStore && bins == 3u) {
+        bool nan = false;
 #pragma unroll
-      for (int i = 0; i < ZL; ++i) acc[q][i] = es != 0.0f ? acc[q][i] * es : 0.0f;
-      fp_finish<S, float, Z, MODE, O>(b, sc, out, at * g.nz + zs.z0, zs, acc[q], red, nullptr);
+        for (int i = 0; i < ZL; ++i) nan = nan || acc[0][i] != acc[0][i] || acc[1][i] != acc[1][i];
+        if (__any_sync(0xffffffffu, nan)) {
+          bins = 1u;
+          continue;
+        }
+      }
+      SIPO_DCHECK(zs.z0 + zs.at(Z::NG - 1) + Z::G - 1 < g.nz, 0);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (!((live & bins) >> q & 1u) || (Z::kRagged && zs.fresh == 0u)) continue;
+        const size_t at = (size_t)k * g.nd + j0 + q;
+        const float es = g.es ? g.es[at] : 1.0f;
+#pragma unroll
+        for (int i = 0; i < ZL; ++i) acc[q][i] = es != 0.0f ? acc[q][i] * es : 0.0f;
+        fp_finish<S, float, Z, MODE, O>(b, sc, out, at * g.nz + zs.z0, zs, acc[q], red, nullptr);
+      }
+      bins = bins == 1u ? 2u : 0u;
     }
   }
 }
