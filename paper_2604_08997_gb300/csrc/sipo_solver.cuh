@@ -296,6 +296,16 @@ __device__ __forceinline__ void dual_update(const Bufs<S, C>& b, const StepScala
   }
 }
 
+// How many neighbouring values of a ray the check step's sums add in the compute
+// type before they go to FP64: whole groups of four (all of a lane's values where
+// z columns are whole tiles of 256), else one, as narrower groups also serve
+// columns that are not whole groups of four.  The sums of a check, and with them
+// its restart and stop decisions, then do not depend on the z form.
+template <typename C, typename Z>
+constexpr int check_fold() {
+  return sizeof(C) == 8 || !Z::kRagged ? Z::ZL : (Z::G == 4 ? 4 : 1);
+}
+
 // ----------------------------------------------------------- primal update
 // One z-vector of rays with g = A q already formed.  CHECK = false: Halpern
 // step fused; CHECK = true: writes y+ and the restart distances (red[0..1]).
@@ -312,7 +322,7 @@ __device__ __forceinline__ void primal_update(const Bufs<S, C>& b, const StepSca
   load_owned<Z>(b.y + base, zs, y);
   load_owned<Z>(b.y0 + base, zs, y0);
   const C w = sc.w;
-  C a0 = C(0), a1 = C(0);  // restart distances of this z-vector (compute type)
+  C a0 = C(0), a1 = C(0);  // restart distances of check_fold values
 #pragma unroll
   for (int i = 0; i < ZL; ++i) {
     const C tau = col[i] > C(0) ? C(kEta) / (sc.omega * col[i]) : C(0);
@@ -326,11 +336,12 @@ __device__ __forceinline__ void primal_update(const Bufs<S, C>& b, const StepSca
       const C dx = y[i] - yp, dz = yp - y0[i];
       a0 += col[i] * dx * dx;
       a1 += col[i] * dz * dz;
+      if ((i + 1) % check_fold<C, Z>() == 0) {
+        red[0] += double(a0);
+        red[1] += double(a1);
+        a0 = a1 = C(0);
+      }
     }
-  }
-  if constexpr (CHECK) {
-    red[0] += double(a0);
-    red[1] += double(a1);
   }
   store_owned<Z>(b.ybar + base, zs, yb);
   if constexpr (!CHECK) {
@@ -389,8 +400,8 @@ __device__ __forceinline__ void resid_update(const Bufs<S, C>& b, size_t base, c
   load_owned<Z>(b.col + base, zs, col);
   load_owned<Z>(b.g0 + base, zs, g0);
   load_owned<Z>(b.gc + base, zs, gc);
-  // sums of one z-vector in the compute type, folded into FP64 once per
-  // vector (as in the check-step dual update)
+  // sums of check_fold values in the compute type, then FP64 (as in the
+  // check-step dual update)
   C a0 = C(0), a1 = C(0), a2 = -CUDART_INF_F, a3 = -CUDART_INF_F;
 #pragma unroll
   for (int i = 0; i < ZL; ++i) {
@@ -402,9 +413,12 @@ __device__ __forceinline__ void resid_update(const Bufs<S, C>& b, size_t base, c
       a2 = a2 > d0 ? a2 : d0;
       a3 = a3 > dc ? a3 : dc;
     }
+    if ((i + 1) % check_fold<C, Z>() == 0) {
+      red[0] += double(a0);
+      red[1] += double(a1);
+      a0 = a1 = C(0);
+    }
   }
-  red[0] += double(a0);
-  red[1] += double(a1);
   red[2] = fmax(red[2], double(a2));
   red[3] = fmax(red[3], double(a3));
   store_owned<Z>(b.gp + base, zs, g);
