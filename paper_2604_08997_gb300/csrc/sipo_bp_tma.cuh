@@ -22,7 +22,7 @@
 //
 // Waits are bounded: one that outlives kWaitCycles sets the context's fault word
 // (tiles.fault, read by the host) and the block's abort flag, on which every wait
-// ends; the copying warp then waits (bounded) for its copies in flight.
+// ends; the copying warp waits (bounded) for its last copies before it ends.
 #pragma once
 
 #include <cuda.h>
@@ -225,8 +225,9 @@ k_backproject_tma(const Geo<float> g, const __grid_constant__ CUtensorMap tmap, 
         }
       }
     }
-    if (lane == 0 && *abort_flag) {
-      // copies in flight write this block's shared memory: wait for them (bounded)
+    if (lane == 0) {
+      // copies in flight write this block's shared memory: wait for them (bounded),
+      // also where a reading warp gives up after the last one was issued
       for (unsigned s = seq > kBtStages ? seq - kBtStages : 0; s < seq; ++s)
         mbar_wait(full + s % kBtStages, (s / kBtStages) & 1u);
     }
