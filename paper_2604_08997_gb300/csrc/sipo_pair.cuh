@@ -8,7 +8,7 @@
 // a zero weight leaves a sum of finite values unchanged, so the sums are those of
 // k_project bit for bit.  An infinite or NaN voxel would reach the other bin as
 // 0 * inf: the plain operator sums a pair that came out NaN again, one bin at a
-// time.  (Four bins a warp, without zero weights through 13 line shapes, moved even
+// time (fp2_again).  (Four bins a warp, without zero weights through 13 line shapes, moved even
 // less but was slower: 16 to 24 warps an SM could not cover a line's chain of
 // table, jump, loads and multiply-adds.)
 //
@@ -37,7 +37,6 @@ struct PairList {
 struct PairRay {
   float c, s, inv_a, h;  // h: half the candidate window with its margin
   int k, j;
-  unsigned bins;         // bit 0: bin j is summed, bit 1: bin j + 1
   bool spread;           // per-bin line ranges apply (flags outside the vial)
   int2 ra, rb;           // line ranges of bins j and j + 1
 };
@@ -69,8 +68,8 @@ __device__ __forceinline__ int fp2_line_taps(const Geo<float>& g, const NeedBits
   const float f0 = ROWS ? cf - g.cx : cf - g.cy;
   float eline = 1.0f;
   if (g.ex) eline = ROWS ? g.ey[(size_t)ray.k * g.ny + line] : g.ex[(size_t)ray.k * g.nx + line];
-  const bool in_a = (ray.bins & 1u) && (!ray.spread || (line >= ray.ra.x && line <= ray.ra.y));
-  const bool in_b = (ray.bins & 2u) && (!ray.spread || (line >= ray.rb.x && line <= ray.rb.y));
+  const bool in_a = !ray.spread || (line >= ray.ra.x && line <= ray.ra.y);
+  const bool in_b = !ray.spread || (line >= ray.rb.x && line <= ray.rb.y);
   int nt = 0;
 #pragma unroll
   for (int m = 0; m < kPairVox; ++m) {
@@ -155,11 +154,45 @@ __device__ __forceinline__ void fp2_walk(const Geo<float>& g, const SI* vz, cons
   }
 }
 
+// The plain operator's bins j0 and j0 + 1 of view k one after the other, by the
+// per-ray walk, written to out.  Out of line, as it runs only where a sum is NaN:
+// 96 x 90 x 96, 391 views took 87.8 us so, 90.5 us with the pair's own loop run again,
+// 97 us with these walks inside the kernel (86.5 us without the check); 128^2 x 130, 360
+// views 224 us, 247 us with the loop run again.
+template <typename SI, typename Z, typename O>
+__device__ __noinline__ void fp2_again(const Geo<float>* gp, const SI* vol, O* out, int k, int j0, int tz,
+                                       PairList* list) {
+  static_assert(sizeof(TapList<float>) <= sizeof(PairList), "list of a ray");
+  const Geo<float>& g = *gp;
+  TapList<float>& tl = *reinterpret_cast<TapList<float>*>(list);
+  const float c = g.cs[2 * k], s = g.cs[2 * k + 1];
+  const bool rows = fabsf(c) >= fabsf(s);
+  ZSpan<Z> zs;
+  zs.init(g.nz, tz);
+  const SI* vz = vol + zs.z0;
+  for (int j = j0; j < min(j0 + 2, g.nd); ++j) {
+    const size_t at = (size_t)k * g.nd + j;
+    const float es = g.es ? g.es[at] : 1.0f;
+    float acc[Z::ZL];
+#pragma unroll
+    for (int i = 0; i < Z::ZL; ++i) acc[i] = 0.0f;
+    if (es != 0.0f) {
+      int lo = 0, hi = (rows ? g.ny : g.nx) - 1;
+      fp_ray_span<float>(g, float(j) - g.off, c, s, rows, lo, hi);
+      if (rows) fp_walk<true, false, Z, SI, float>(g, vz, NeedBits{}, false, k, float(j), c, s, lo, hi, zs, tl, acc);
+      else fp_walk<false, false, Z, SI, float>(g, vz, NeedBits{}, false, k, float(j), c, s, lo, hi, zs, tl, acc);
+#pragma unroll
+      for (int i = 0; i < Z::ZL; ++i) acc[i] *= es;
+    }
+    if (!Z::kRagged || zs.fresh != 0u) store_owned<Z>(out + at * g.nz + zs.z0, zs, acc);
+  }
+}
+
 // Tile: aw consecutive views x 8 / aw consecutive bin pairs, one z tile; a warp
 // sums one pair of one view.  Other arguments as k_project.
 template <typename SI, typename S, typename Z, int MODE, typename O>
 __global__ void __launch_bounds__(kThreads, 4)
-k_project_pair(const Geo<float> g, const SI* __restrict__ vol, const Bufs<S, float> b, O* __restrict__ out,
+k_project_pair(const __grid_constant__ Geo<float> g, const SI* __restrict__ vol, const Bufs<S, float> b, O* __restrict__ out,
                const uint8_t* __restrict__ act_col, const NeedBits nb, const int2* __restrict__ rspan, int aw) {
   static_assert(MODE == kFpStore || MODE == kFpPrimal, "modes without reductions");
   const bool use_bits = nb.rows != nullptr;
@@ -219,39 +252,35 @@ k_project_pair(const Geo<float> g, const SI* __restrict__ vol, const Bufs<S, flo
     zs.init(g.nz, tz);
     const SI* vz = vol + zs.z0;
     PairList& tl = taps[warp];
-    // both bins together; a pair that came out NaN again, one after the other
-    for (unsigned bins = 3u; bins != 0u;) {
-      ray.bins = bins;
-      float acc[2][ZL];
+    float acc[2][ZL];
 #pragma unroll
-      for (int i = 0; i < ZL; ++i) acc[0][i] = acc[1][i] = 0.0f;
-      if (rows) {
-        if (j0 >= 2) fp2_walk<true, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
-        else fp2_walk<true, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
-      } else {
-        if (j0 >= 2) fp2_walk<false, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
-        else fp2_walk<false, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+    for (int i = 0; i < ZL; ++i) acc[0][i] = acc[1][i] = 0.0f;
+    if (rows) {
+      if (j0 >= 2) fp2_walk<true, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+      else fp2_walk<true, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+    } else {
+      if (j0 >= 2) fp2_walk<false, true, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+      else fp2_walk<false, false, Z, SI>(g, vz, nb, use_bits, ray, lo, hi, zs, tl, acc);
+    }
+    if constexpr (MODE == kFpStore) {
+      bool nan = false;
+#pragma unroll
+      for (int i = 0; i < ZL; ++i) nan = nan || acc[0][i] != acc[0][i] || acc[1][i] != acc[1][i];
+      if (__any_sync(0xffffffffu, nan)) {
+        fp2_again<SI, Z, O>(&g, vol, out, k, j0, tz, &tl);
+        continue;
       }
-      if (MODE == kFpStore && bins == 3u) {
-        bool nan = false;
+    }
+    if (Z::kRagged && zs.fresh == 0u) continue;
+    SIPO_DCHECK(zs.z0 + zs.at(Z::NG - 1) + Z::G - 1 < g.nz, 0);
 #pragma unroll
-        for (int i = 0; i < ZL; ++i) nan = nan || acc[0][i] != acc[0][i] || acc[1][i] != acc[1][i];
-        if (__any_sync(0xffffffffu, nan)) {
-          bins = 1u;
-          continue;
-        }
-      }
-      SIPO_DCHECK(zs.z0 + zs.at(Z::NG - 1) + Z::G - 1 < g.nz, 0);
+    for (int q = 0; q < 2; ++q) {
+      if (!((live >> q) & 1u)) continue;
+      const size_t at = (size_t)k * g.nd + j0 + q;
+      const float es = g.es ? g.es[at] : 1.0f;
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        if (!((live & bins) >> q & 1u) || (Z::kRagged && zs.fresh == 0u)) continue;
-        const size_t at = (size_t)k * g.nd + j0 + q;
-        const float es = g.es ? g.es[at] : 1.0f;
-#pragma unroll
-        for (int i = 0; i < ZL; ++i) acc[q][i] = es != 0.0f ? acc[q][i] * es : 0.0f;
-        fp_finish<S, float, Z, MODE, O>(b, sc, out, at * g.nz + zs.z0, zs, acc[q], red, nullptr);
-      }
-      bins = bins == 1u ? 2u : 0u;
+      for (int i = 0; i < ZL; ++i) acc[q][i] = es != 0.0f ? acc[q][i] * es : 0.0f;
+      fp_finish<S, float, Z, MODE, O>(b, sc, out, at * g.nz + zs.z0, zs, acc[q], red, nullptr);
     }
   }
 }
