@@ -28,6 +28,7 @@
 #include "sipo_psf.cuh"
 #include "sipo_response.cuh"
 #include "sipo_schedule.h"
+#include "sipo_tiles.h"
 
 namespace sipo {
 namespace {
@@ -893,8 +894,8 @@ struct Solver final : SolverBase {
     return list;
   }
 
-  // Chooses the tiles by shape and target alone (sums do not depend on timing)
-  // and lists the solver's.
+  // Chooses the tiles by shape and target alone (sums depend neither on timing
+  // nor on the device) and lists the solver's.
   void choose_bp_tiles() {
     if constexpr (sizeof(C) == 8) return;
     int T = 1;
@@ -903,18 +904,9 @@ struct Solver final : SolverBase {
     std::vector<uint8_t> cols(size_t(nx) * ny);
     ck(cudaMemcpyAsync(cols.data(), need, cols.size(), cudaMemcpyDeviceToHost, stream), "need");
     ck(cudaStreamSynchronize(stream), "need");
-    // Tiles of 8 rows where they cover the SMs one and a half times, else of 2: a
-    // tile lasts as long as its views, and on a small part more of them, on more
-    // SMs, is what is left to gain.  Staged rows, solver step, ms with 8 / 4 / 2 rows
-    // (tiles of 8): 64^3 x 180 (41) 0.060 / 0.057 / 0.054; 112^3 x 333 (134) 0.111 /
-    // 0.103 / 0.101; 160^3 x 300 (164) 0.136 / 0.125 / 0.126; 192^3 x 300 (286) 0.158 /
-    // 0.247 / 0.241; 256^3 x 360 (490) 0.338 / 0.422 / 0.505.
-    const long long want = 3LL * device_sms() / 2;
     std::vector<int> list = bp_tile_list(cols, 8);
-    if ((long long)list.size() * nzc < want) {
-      bpt.rows = 2;
-      list = bp_tile_list(cols, 2);
-    }
+    bpt.rows = bp_rows(double(list.size()) * double(nzc));
+    if (bpt.rows != 8) list = bp_tile_list(cols, bpt.rows);
     int* d = dalloc<int>(list.size());
     ck(cudaMemcpyAsync(d, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, stream), "tiles");
     ck(cudaStreamSynchronize(stream), "tiles");
@@ -924,14 +916,11 @@ struct Solver final : SolverBase {
     const double share = vial_r > 0 ? std::min(1.0, 3.14159265 * vial_r * vial_r / (double(nx) * ny)) : 1.0;
     auto tiles = [&](int rows) { return share * ((nx + kBp2NV - 1) / kBp2NV) * ((ny + rows - 1) / rows) * double(nzc); };
     if (bp_staged(nz)) {
-      if (tiles(8) < double(want)) bpt_all.rows = 2;
+      bpt_all.rows = bp_rows(tiles(8));
     } else {
-      // without staged rows the chain of a warp's views is long: shared by up to
-      // eight warps until there are 1.75 rounds of the 3 resident blocks an SM.
-      // 128^2 x 130 x 360 (122 tiles of 8 rows), solver step, ms by split 0, 1, 2, 3:
-      // 0.199, 0.116, 0.079, 0.087.
-      while (bpt_all.split < 3 && tiles(8 >> bpt_all.split) < 1.75 * 3 * device_sms()) ++bpt_all.split;
-      bpt_all.rows = 8 >> bpt_all.split;
+      const BpPlan p = bp_split(tiles);
+      bpt_all.rows = p.rows;
+      bpt_all.split = p.split;
     }
   }
 

@@ -20,7 +20,8 @@ constexpr int kWarps = kThreads / 32;
 // Grid of every reducing kernel: 8 blocks per SM of a 152-SM GB300.  It is a
 // constant on purpose: the FP64 reductions sum one partial per block in block
 // order, so a fixed grid keeps every solve bit-reproducible from one device to
-// another whatever its SM count; the grid-stride loops stay correct on any.
+// another whatever its SM count; the grid-stride loops stay correct on any.  (The
+// tiles that enter the sums are chosen against the same number, see sipo_tiles.h.)
 constexpr int kRedBlocks = 1216;
 
 // Streaming multiprocessors of the current device (cudaDeviceProp
