@@ -915,7 +915,7 @@ struct Solver final : SolverBase {
     // the plain operator: every tile, of which about `share` have work
     const double share = vial_r > 0 ? std::min(1.0, 3.14159265 * vial_r * vial_r / (double(nx) * ny)) : 1.0;
     auto tiles = [&](int rows) { return share * ((nx + kBp2NV - 1) / kBp2NV) * ((ny + rows - 1) / rows) * double(nzc); };
-    if (bp_staged(nz)) {
+    if (bp_staged<C>(nz)) {
       bpt_all.rows = bp_rows(tiles(8));
     } else {
       const BpPlan p = bp_split(tiles);
@@ -1226,6 +1226,10 @@ struct Solver final : SolverBase {
     solved = false;
   }
 
+  // Entry of the plain operator, whose sinograms are in the compute type: staged
+  // rows also where those of the storage type cannot be (bf16, nz = 4 mod 8).
+  int plain_tile() const { return sizeof(C) == 4 && tol.tile_cfg < 0 && bp_staged<C>(nz) ? 5 : bp_nv; }
+
   // Tile table (kBpTiles entries, see launch_backproject).  tile_cfg >= 0
   // selects an entry; -1 times a few un-captured iterations of each entry with
   // CUDA events (backprojection phase) and keeps the fastest.
@@ -1236,7 +1240,7 @@ struct Solver final : SolverBase {
       return;
     }
     if (bp_flat<C>(nz)) return;  // no tiles to choose from
-    if (sizeof(C) == 4 && bp_staged(nz)) {
+    if (sizeof(C) == 4 && bp_staged<S>(nz)) {
       // staged rows were the fastest entry on every size measured (64^3 to 384^3,
       // FP32 and BF16 storage: 0.60 to 0.97 of the best of entries 3 and 4)
       bp_nv = 5;
@@ -1545,11 +1549,11 @@ struct Solver final : SolverBase {
     if (psf) {
       ensure_temps();
       launch_backproject<C, C, C, kBpStore, C>(g, static_cast<const C*>(sino), Bufs<C, C>{}, t3, nullptr, s, bpt_all,
-                                               bp_nv);
+                                               plain_tile());
       psf3<C, C>(t3, static_cast<C*>(vol), t1, t2, -1, s);
     } else {
       launch_backproject<C, C, C, kBpStore, C>(g, static_cast<const C*>(sino), Bufs<C, C>{},
-                                               static_cast<C*>(vol), nullptr, s, bpt_all, bp_nv);
+                                               static_cast<C*>(vol), nullptr, s, bpt_all, plain_tile());
     }
     count(1);
     ck(cudaGetLastError(), "backproject");
@@ -1575,7 +1579,7 @@ struct Solver final : SolverBase {
     // order shows in them
     const BpTiles whole{nullptr, 0, bpt.rows, 0, bpt.fault};
     launch_backproject<C, C, C, kBpStore, C>(geo(), static_cast<const C*>(sino), Bufs<C, C>{}, tvol, nullptr,
-                                             s, whole, bp_nv);
+                                             s, whole, plain_tile());
     count(1);
     for (int a = 0; a < 3; ++a) {
       grad[a] = 0.0;

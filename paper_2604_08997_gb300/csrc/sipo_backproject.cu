@@ -100,7 +100,7 @@ void launch_backproject(const Geo<C>& g, const SI* sino, const Bufs<S, C>& b, O*
     return;
   }
   if constexpr (std::is_same<C, float>::value) {
-    if (tile >= 5 && bp_staged(g.nz)) {
+    if (tile >= 5 && bp_staged<SI>(g.nz)) {
       auto go = [&](auto ng) {
         constexpr int NG = decltype(ng)::value;
         return tiles.rows == 8 ? launch_bp_tma<SI, S, NG, 8, MODE, O>(g, sino, b, out, need, tiles, stream)

@@ -59,8 +59,10 @@ template <typename C> inline bool fp_flat(const Geo<C>& g) {
 }
 template <typename C> inline bool bp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 9 : 12); }
 
-// Whether the staged backprojector covers this z extent.
-inline bool bp_staged(int nz) { return nz % 4 == 0; }
+// Whether the staged backprojector covers sinograms of SI with this z extent: a lane
+// takes groups of four values, and a tensor map needs strides of whole 16 bytes
+// (bf16: nz a multiple of 8).
+template <typename SI> inline bool bp_staged(int nz) { return nz % 4 == 0 && nz * sizeof(SI) % 16 == 0; }
 
 // Group size G of the z layout (elements of C in 16 bytes).
 template <typename C> constexpr int z_group() { return 16 / int(sizeof(C)); }

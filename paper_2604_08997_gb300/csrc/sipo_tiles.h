@@ -20,7 +20,9 @@ struct BpPlan {
 // is left to gain.  Staged rows, solver step, ms with 8 / 4 / 2 rows (tiles of 8):
 // 64^3 x 180 (41) 0.060 / 0.057 / 0.054; 112^3 x 333 (134) 0.111 / 0.103 / 0.101; 160^3 x
 // 300 (164) 0.136 / 0.125 / 0.126; 192^3 x 300 (286) 0.158 / 0.247 / 0.241; 256^3 x 360
-// (490) 0.338 / 0.422 / 0.505.
+// (490) 0.338 / 0.422 / 0.505.  Rows read in place, 8 / 2 rows: 64^2 x 66 x 180 0.090 /
+// 0.088; 128^2 x 130 x 360 0.174 / 0.170; 160^2 x 162 x 300 0.152 / 0.148; BF16 160^2 x 164 x
+// 300 0.172 / 0.153.
 inline int bp_rows(double tiles_of_8) { return tiles_of_8 < 3 * kPlanSms / 2 ? 2 : 8; }
 
 // The plain operator with rows read in place: the chain of a warp's views is long,
