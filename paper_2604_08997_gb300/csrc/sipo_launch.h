@@ -77,34 +77,51 @@ inline int z_group_for(int nz, const A* a, const B* b) {
   return G;
 }
 
-// Calls f(ZForm) with the z form for extent nz and groups of at most gmax values
-// (see ZForm): the form with the least tiles * time per tile.  The times are the
-// measured ones of the solver's projector and backprojector (mean of both, 240^2 x
-// 512 and 160^2 x 48, 300 views, FP32) relative to the form {4, 1}; they follow
-// the 16-, 8- or 4-byte loads of a tap plus its fixed part.  E.g. 160^2 x 160,
-// projector: {2, 3} 0.098 ms, {4, 2} 0.113, {4, 1} 0.152.  Double precision
-// keeps two forms of pairs, and single values up to nz = 32, where pairs leave
-// half of the lanes idle (200^2 x 16: 2.70 ms, single 1.81).  widest: only groups
-// of gmax values (the solver's sums are formed group by group).
+// Single-precision z forms and their time per tile: the measured ones of the solver's
+// projector and backprojector (mean of both, 240^2 x 512 and 160^2 x 48, 300 views)
+// relative to the form {4, 1}; they follow the 16-, 8- or 4-byte loads of a tap plus
+// its fixed part.  E.g. 160^2 x 160, projector: {2, 3} 0.098 ms, {4, 2} 0.113, {4, 1} 0.152.
+// The last one is {4, 2} where nz is whole tiles of 256.
+struct ZCost { int G, NG; double time; };
+constexpr int kZForms = 11;
+constexpr ZCost kZCosts[kZForms] = {{4, 2, 1.5}, {4, 1, 1.0}, {2, 4, 1.63}, {2, 3, 1.3}, {2, 2, 1.09},
+                                    {2, 1, 0.87}, {1, 8, 2.2}, {1, 4, 1.17}, {1, 2, 0.96}, {1, 1, 0.76}, {4, 2, 1.25}};
+
+// Warps that the projector keeps resident on a GB300 (32 an SM).  Below that a
+// launch lasts as long as one warp, whatever their number.
+constexpr double kFpSlots = 152.0 * 32.0;
+
+// The form (index of kZCosts) with the least time, for groups of at most gmax values
+// (widest: of exactly gmax, as the solver's sums are formed group by group).  warps:
+// warps per z tile of a launch that may leave slots empty, where a narrower form on
+// more warps takes less time; 0: tiles * time per tile.  *cost: its time.
+inline int z_form(int nz, int gmax, bool widest, double warps, double* cost) {
+  int best = 9;
+  *cost = 1e300;
+  for (int i = 0; i < kZForms; ++i) {
+    const ZCost& f = kZCosts[i];
+    if ((widest ? f.G != gmax : f.G > gmax) || (i == 10 && nz % 256 != 0) || (i == 0 && nz % 256 == 0)) continue;
+    const int T = 32 * f.G * f.NG;
+    const double tiles = (nz + T - 1) / T, t = warps > 0 ? warps * tiles : tiles;
+    const double c = (t > kFpSlots || warps <= 0 ? t : kFpSlots) * f.time;
+    if (c < *cost) { *cost = c; best = i; }
+  }
+  return best;
+}
+
+// Calls f(ZForm) with the form chosen for extent nz and groups of at most gmax values
+// (see z_form).  Double precision keeps two forms of pairs, and single values up to
+// nz = 32, where pairs leave half of the lanes idle (200^2 x 16: 2.70 ms, single 1.81).
 template <typename C, typename F>
-inline void with_z_form(int nz, int gmax, F&& f, bool widest = false) {
+inline void with_z_form(int nz, int gmax, F&& f, bool widest = false, double warps = 0.0) {
   if constexpr (sizeof(C) == 8) {
     if (gmax >= 2 && nz % 128 == 0) f(ZForm<2, 2, false>{});
     else if (gmax >= 2 && nz > 32) f(ZForm<2, 1, true>{});
     else f(ZForm<1, 1, true>{});
   } else {
-    if (gmax >= 4 && nz % 256 == 0) return f(ZForm<4, 2, false>{});
-    struct Cost { int G, NG; double time; };
-    constexpr Cost forms[10] = {{4, 2, 1.5}, {4, 1, 1.0}, {2, 4, 1.63}, {2, 3, 1.3}, {2, 2, 1.09},
-                                {2, 1, 0.87}, {1, 8, 2.2}, {1, 4, 1.17}, {1, 2, 0.96}, {1, 1, 0.76}};
-    int best = 9;
-    double least = 1e300;
-    for (int i = 0; i < 10; ++i) {
-      const int T = 32 * forms[i].G * forms[i].NG;
-      const double cost = ((nz + T - 1) / T) * forms[i].time;
-      if ((widest ? forms[i].G == gmax : forms[i].G <= gmax) && cost < least) { least = cost; best = i; }
-    }
-    switch (best) {
+    double cost;
+    if (warps <= 0 && gmax >= 4 && nz % 256 == 0) return f(ZForm<4, 2, false>{});
+    switch (z_form(nz, gmax, widest, warps, &cost)) {
       case 0: return f(ZForm<4, 2, true>{});
       case 1: return f(ZForm<4, 1, true>{});
       case 2: return f(ZForm<2, 4, true>{});
@@ -114,9 +131,41 @@ inline void with_z_form(int nz, int gmax, F&& f, bool widest = false) {
       case 6: return f(ZForm<1, 8, true>{});
       case 7: return f(ZForm<1, 4, true>{});
       case 8: return f(ZForm<1, 2, true>{});
-      default: return f(ZForm<1, 1, true>{});
+      case 9: return f(ZForm<1, 1, true>{});
+      default: return f(ZForm<4, 2, false>{});
     }
   }
+}
+
+// How a projection without sums (the plain operator, the solver's step) runs in
+// single precision; every choice gives the same sums, bit for bit.
+struct FpPlan {
+  bool flat;     // lanes over bins (nz <= 8)
+  bool pair;     // two bins a warp, else one
+  double warps;  // per z tile, for with_z_form
+};
+
+// Two bins a warp move fewer columns, one bin a warp makes twice the warps, each done
+// in 0.65 of the time; the flat form costs 1.75 a warp and is full at 1500 warps.  The
+// three figures are fitted to 296 projections (48^2 to 320^2, nz 1 to 384, 4 to 128
+// views, every form timed): the choice is 2% behind the best of all on average,
+// 26% at worst.  Pairs and the widest form everywhere were 36% behind: 200^2 x 200,
+// 8 views, 90 us, now 35; 64^2 x 130, 32 views 24.8 -> 16.6; flat slices of 200^2, 8
+// views 31 -> 20.7.
+template <typename C>
+inline FpPlan fp_plan(const Geo<C>& g, int gmax, bool flat_ok) {
+  const double rays = double(g.na) * g.nd, pairs = double(g.na) * ((g.nd + 1) / 2);
+  double ray_cost, pair_cost;
+  z_form(g.nz, gmax, false, rays, &ray_cost);
+  z_form(g.nz, gmax, false, pairs, &pair_cost);
+  ray_cost *= 0.65;
+  const double z_cost = ray_cost < pair_cost ? ray_cost : pair_cost;
+  const double fw = double(g.na) * ((g.nd + 30) / 31) * g.nz;
+  FpPlan p;
+  p.flat = flat_ok && 1.75 * (fw > 1500.0 ? fw : 1500.0) < z_cost;
+  p.pair = pair_cost <= ray_cost;
+  p.warps = p.pair ? pairs : rays;
+  return p;
 }
 
 }  // namespace sipo

@@ -51,20 +51,35 @@ void launch_project(const Geo<C>& g, const SI* vol, const Bufs<S, C>& b, O* out,
                     const int2* rspan) {
   // the slice-mode certificate keeps one 8-byte maximum per z in shared memory
   const size_t dyn = MODE == kFpCertZ ? size_t(g.nz) * sizeof(unsigned long long) : 0;
-  if (fp_flat<C>(g)) {
+  const int gmax = z_group_for<C>(g.nz, vol, out);
+  // the modes of the check step have sums, whose order follows the form: they keep
+  // one rule by extent (they run once a period).  bf16 steps always take pairs: the
+  // compiler rounds their Halpern step in another order from kernel to kernel, and
+  // bf16 iterates show it (2e-2 after two periods).
+  constexpr bool kPairs = sizeof(C) == 4 && (MODE == kFpPrimal || MODE == kFpStore);
+  constexpr bool kPlanned = kPairs && (MODE == kFpStore || sizeof(S) == 4);
+  bool flat = fp_flat<C>(g);
+  FpPlan plan{flat, true, 0.0};
+  if constexpr (kPlanned) {
+    plan = fp_plan<C>(g, gmax, flat);
+    flat = plan.flat;
+  }
+  if (flat) {
     // a solver's input vanishes outside its flagged columns; those may lie
     // outside the vial where a PSF spreads them
     const bool wide = nb.rows != nullptr && g.r2i >= 0 && nb.spread;
     k_project_flat<SI, S, C, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, rspan, wide);
     return;
   }
-  with_z_form<C>(g.nz, z_group_for<C>(g.nz, vol, out), [&](auto form) {
+  with_z_form<C>(g.nz, gmax, [&](auto form) {
     using Z = decltype(form);
-    if constexpr (sizeof(C) == 4 && (MODE == kFpPrimal || MODE == kFpStore)) {
-      // two bins a warp, the same sums; the modes of the check step keep one
-      // (they run once a period).  4 views a tile: 0.344 / 0.560 ms on two targets at
-      // 256^3 x 360, 8 views 0.321 / 0.587; 96^3 x 391 0.0529, 0.0552.
-      k_project_pair<SI, S, Z, MODE, O><<<kRedBlocks, kThreads, 0, stream>>>(g, vol, b, out, act_col, nb, rspan, 4);
+    if constexpr (kPairs) {
+      // 4 views a tile: 0.344 / 0.560 ms on two targets at 256^3 x 360, 8 views 0.321 / 0.587;
+      // 96^3 x 391 0.0529, 0.0552.  One view a tile on few warps: the same within 4%.
+      if (!kPlanned || plan.pair)
+        k_project_pair<SI, S, Z, MODE, O><<<kRedBlocks, kThreads, 0, stream>>>(g, vol, b, out, act_col, nb, rspan, 4);
+      else if constexpr (kPlanned)
+        k_project<SI, S, C, Z, MODE, O><<<kRedBlocks, kThreads, 0, stream>>>(g, vol, b, out, act_col, nb, rspan, 4);
     } else {
       // Views per tile: 4 where every block has several tiles to even out, else 1.
       // 256^3 x 360 (9.5 tiles a block): 0.420 ms with 1, 0.394 with 2, 0.360 with 4,
@@ -74,7 +89,7 @@ void launch_project(const Geo<C>& g, const SI* vol, const Bufs<S, C>& b, O* out,
       const int aw = tiles >= 8LL * kRedBlocks ? 4 : 1;
       k_project<SI, S, C, Z, MODE, O><<<kRedBlocks, kThreads, dyn, stream>>>(g, vol, b, out, act_col, nb, rspan, aw);
     }
-  });
+  }, false, plan.warps);
 }
 
 void launch_need_bits(const uint8_t* need, uint32_t* rows, uint32_t* cols, int nx, int ny, int wr, int wc,

@@ -330,7 +330,9 @@ __device__ __forceinline__ void primal_update(const Bufs<S, C>& b, const StepSca
     yp = rnd<S, C>(yp > C(0) ? yp : C(0));
     yb[i] = rnd<S, C>(C(2) * yp - y[i]);
     if constexpr (!CHECK) {
-      yo[i] = w * yb[i] + (C(1) - w) * y0[i];
+      // one rounding order in every kernel, as several serve a step (bf16: one kernel)
+      if constexpr (sizeof(S) != 2) yo[i] = fma(C(1) - w, y0[i], w * yb[i]);
+      else yo[i] = w * yb[i] + (C(1) - w) * y0[i];
     } else {
       yo[i] = yp;
       const C dx = y[i] - yp, dz = yp - y0[i];
