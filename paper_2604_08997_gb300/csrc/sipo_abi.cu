@@ -918,7 +918,7 @@ struct Solver final : SolverBase {
     if (bp_staged<C>(nz)) {
       bpt_all.rows = bp_rows(tiles(8));
     } else {
-      const BpPlan p = bp_split(tiles);
+      const BpPlan p = bp_split(na, tiles);
       bpt_all.rows = p.rows;
       bpt_all.split = p.split;
     }
@@ -1226,9 +1226,12 @@ struct Solver final : SolverBase {
     solved = false;
   }
 
-  // Entry of the plain operator, whose sinograms are in the compute type: staged
-  // rows also where those of the storage type cannot be (bf16, nz = 4 mod 8).
-  int plain_tile() const { return sizeof(C) == 4 && tol.tile_cfg < 0 && bp_staged<C>(nz) ? 5 : bp_nv; }
+  // Entry of the plain operator, which is not the one that the solver step was timed
+  // for: its sinograms are in the compute type (staged rows also where those of the
+  // storage type cannot be, bf16 and nz = 4 mod 8), and in place it has every column
+  // of the vial, where 3 blocks an SM are faster: us, entry 3 / 4, 128^2 x 13 x 180 100 /
+  // 84; 200^2 x 31 x 180 233 / 186; 200^2 x 66 x 180 287 / 232; 320^2 x 13 x 180 526 / 392.
+  int plain_tile() const { return sizeof(C) == 8 || tol.tile_cfg >= 0 ? bp_nv : bp_staged<C>(nz) ? 5 : 4; }
 
   // Tile table (kBpTiles entries, see launch_backproject).  tile_cfg >= 0
   // selects an entry; -1 times a few un-captured iterations of each entry with

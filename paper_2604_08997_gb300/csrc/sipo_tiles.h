@@ -28,11 +28,13 @@ inline int bp_rows(double tiles_of_8) { return tiles_of_8 < 3 * kPlanSms / 2 ? 2
 // The plain operator with rows read in place: the chain of a warp's views is long,
 // so it is shared by up to eight warps until there are 1.75 rounds of the 3 resident
 // blocks an SM.  128^2 x 130 x 360 (122 tiles of 8 rows), ms by split 0, 1, 2, 3:
-// 0.199, 0.116, 0.079, 0.087.  tiles(rows): tiles with work.
+// 0.199, 0.116, 0.079, 0.087.  A warp keeps seven views at least: with fewer the shares
+// cost more to add than they take off the chain (64^2 x 66, 8 views, eight warps 14.4 us,
+// one 10.6).  tiles(rows): tiles with work.
 template <typename F>
-inline BpPlan bp_split(F&& tiles) {
+inline BpPlan bp_split(int views, F&& tiles) {
   BpPlan p{8, 0};
-  while (p.split < 3 && tiles(p.rows) < 1.75 * 3 * kPlanSms) {
+  while (p.split < 3 && (views >> (p.split + 1)) >= 7 && tiles(p.rows) < 1.75 * 3 * kPlanSms) {
     ++p.split;
     p.rows >>= 1;
   }

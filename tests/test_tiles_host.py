@@ -20,9 +20,11 @@ int main() {
   // tiles of 8 rows; twice as many with half the rows
   const double eights[] = {1, 100, 122, 199, 200, 398, 399, 797, 798, 5000};
   for (double n : eights) {
-    const sipo::BpPlan p = sipo::bp_split([&](int rows) { return n * 8 / rows; });
+    const sipo::BpPlan p = sipo::bp_split(180, [&](int rows) { return n * 8 / rows; });
     std::printf("%d:%d ", p.rows, p.split);
   }
+  const int views[] = {1, 8, 13, 14, 27, 28, 55, 56, 60, 400};
+  for (int k : views) std::printf("%d ", sipo::bp_split(k, [](int) { return 1.0; }).split);
   return 0;
 }
 """
@@ -39,7 +41,9 @@ def test_tiles_follow_from_the_shape_alone(tmp_path):
     out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.split()
     assert out[:8] == ["2", "2", "2", "2", "2", "8", "8", "8"]
     # shared until there are 1.75 * 3 * 152 = 798 tiles, by eight warps at most
-    assert out[8:] == ["1:3", "1:3", "1:3", "1:3", "2:2", "2:2", "4:1", "4:1", "8:0", "8:0"]
+    assert out[8:18] == ["1:3", "1:3", "1:3", "1:3", "2:2", "2:2", "4:1", "4:1", "8:0", "8:0"]
+    # seven views a warp at least
+    assert out[18:] == ["0", "0", "0", "1", "1", "2", "2", "3", "3", "3"]
 
 
 def test_the_solver_asks_no_device_for_them():
