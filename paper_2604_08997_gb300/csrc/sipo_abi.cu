@@ -1242,7 +1242,7 @@ struct Solver final : SolverBase {
       bp_nv = tol.tile_cfg;
       return;
     }
-    if (bp_flat<C>(nz)) return;  // no tiles to choose from
+    if (bp_flat<C>(nx, ny, nz)) return;  // no tiles to choose from
     if (sizeof(C) == 4 && bp_staged<S>(nz)) {
       // staged rows were the fastest entry on every size measured (64^3 to 384^3,
       // FP32 and BF16 storage: 0.60 to 0.97 of the best of entries 3 and 4)

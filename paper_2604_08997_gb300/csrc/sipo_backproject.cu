@@ -95,7 +95,7 @@ bool launch_bp_tma(const Geo<float>& g, const SI* sino, const Bufs<S, float>& b,
 template <typename SI, typename S, typename C, int MODE, typename O>
 void launch_backproject(const Geo<C>& g, const SI* sino, const Bufs<S, C>& b, O* out,
                         const uint8_t* need, cudaStream_t stream, const BpTiles& tiles, int tile) {
-  if (bp_flat<C>(g.nz)) {
+  if (bp_flat<C>(g.nx, g.ny, g.nz)) {
     k_backproject_flat<SI, S, C, MODE, O><<<kRedBlocks, kThreads, 0, stream>>>(g, sino, b, out, need);
     return;
   }

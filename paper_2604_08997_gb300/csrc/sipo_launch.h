@@ -46,18 +46,28 @@ template <typename SI, typename S, typename C, int MODE, typename O>
 void launch_backproject(const Geo<C>& g, const SI* sino, const Bufs<S, C>& b, O* out,
                         const uint8_t* need, cudaStream_t stream, const BpTiles& tiles, int tile = 0);
 
-// z extents that take the kernels of sipo_flat.cuh (lanes over bins or voxels):
-// below these the z lanes of the other kernels idle more than the flat ones
-// repeat weights.  200 x 200, 300 views, us, z lanes / flat: single precision,
-// projector 274 / 115 at nz = 4, 277 / 246 at 8, 279 / 349 at 12; backprojector
-// 317 / 149 at 8, 317 / 209 at 12, 319 / 411 at 16; double precision, projector
-// 2696 / 1859 at 4, 2696 / 2738 at 6; backprojector 2387 / 1950 at 8, 2480 / 2879 at 12.
+// Volumes that take the kernels of sipo_flat.cuh (lanes over bins or voxels): at few z
+// values the z lanes of the other kernels idle more than the flat ones repeat
+// weights.  Single precision, 200 x 200, 300 views, us, z lanes / flat: projector 274 / 115
+// at nz = 4, 277 / 246 at 8, 279 / 349 at 12 (fp_plan chooses below that); backprojector
+// 317 / 149 at 8, 317 / 209 at 12, 319 / 411 at 16.
+// Double precision (z lanes: single values, the same at every nz below 32), 180 views,
+// us, z lanes / flat.  Projector: 200 x 200 1427 / 1109 at 3, 1445 at 4; 64 x 64 161 / 165 at
+// 3, 220 at 4; a detector twice the grid, whose outer rays end at once in z lanes, 200 x
+// 200, 60 views 569 / 475 at 2, 690 at 3.  Backprojector: 200 x 200 1190 / 935 at 6, 1248 at 8;
+// 128 x 128 430 / 370 at 6, 454 at 8; 64 x 64, where z lanes of four columns leave warps free,
+// 268 / 138 at 9.
 // The flat projector's candidate window holds up to sides (and detectors) of kFlatSide.
 constexpr int kFlatSide = 16384;
 template <typename C> inline bool fp_flat(const Geo<C>& g) {
-  return g.nz <= (sizeof(C) == 8 ? 5 : 8) && g.nx <= kFlatSide && g.ny <= kFlatSide && g.nd <= kFlatSide;
+  const int side = g.nx > g.ny ? g.nx : g.ny;
+  const int most = sizeof(C) == 4 ? 8 : (g.nd > side + side / 2 ? 2 : 3);
+  return g.nz <= most && side <= kFlatSide && g.nd <= kFlatSide;
 }
-template <typename C> inline bool bp_flat(int nz) { return nz <= (sizeof(C) == 8 ? 9 : 12); }
+template <typename C> inline bool bp_flat(int nx, int ny, int nz) {
+  if (sizeof(C) == 4) return nz <= 12;
+  return nz <= ((nx + 3LL) / 4 * ny >= 24LL * 152 ? 6 : 9);  // 24 warps an SM of z lanes
+}
 
 // Whether the staged backprojector covers sinograms of SI with this z extent: a lane
 // takes groups of four values, and a tensor map needs strides of whole 16 bytes
