@@ -88,6 +88,16 @@ def captured_traffic(workload: str, storage: str, kernel: str):
     return rec[kernel]
 
 
+def kernel_names(storage: str, nz: int, tile_cfg: int):
+    """Backprojector and projector kernels of a solver step on the workloads of this
+    file (2-D slices, or volumes of 64 z values and more, with hundreds of views)."""
+    if nz == 1:
+        return "k_backproject_flat", "k_project_flat"
+    if storage == "f64":
+        return "k_backproject", "k_project"
+    return "k_backproject_tma" if tile_cfg >= 5 else "k_backproject2", "k_project_pair"
+
+
 # ------------------------------------------------------------- distributed
 def dist_env():
     world = int(os.environ.get("WORLD_SIZE", "1"))
@@ -512,8 +522,7 @@ def run_gpu(args, dist, rank, world, device):
     fp_ms = phases["project_primal"]
     tr_bp = captured_traffic(args.workload, args.storage, "backproject")
     tr_fp = captured_traffic(args.workload, args.storage, "project")
-    bp_name = "k_backproject_tma" if res["tile_cfg"] >= 5 else "k_backproject2"
-    fp_name = "k_project" if args.storage == "f64" else "k_project_pair"
+    bp_name, fp_name = kernel_names(args.storage, wl.nz, res["tile_cfg"])
     if bp_ms >= fp_ms:
         dom, dom_ms, taps, traffic = f"{bp_name} (fused dual update)", bp_ms, bp_taps, tr_bp
     else:

@@ -85,3 +85,11 @@ def test_reference_arm_uses_every_host_core(capsys):
         if d["value"] > one["value"]:
             break
     assert d["value"] > one["value"]
+
+
+@pytest.mark.parametrize("storage,nz,tile,names", [
+    ("f64", 1, 0, ("k_backproject_flat", "k_project_flat")), ("f32", 1, 0, ("k_backproject_flat", "k_project_flat")),
+    ("f64", 64, 2, ("k_backproject", "k_project")), ("f32", 256, 5, ("k_backproject_tma", "k_project_pair")),
+    ("bf16", 260, 4, ("k_backproject2", "k_project_pair"))])
+def test_reported_kernels_are_those_of_the_storage_and_extent(storage, nz, tile, names):
+    assert bench.kernel_names(storage, nz, tile) == names
