@@ -452,8 +452,9 @@ const char *sipo_phase_name(int i);
  * Single precision: the row-pattern kernel (4 voxel columns a warp, the rows of
  * each angle in registers, packed FP32 multiply-adds) at 2 blocks/SM (entries 0,
  * 1, 3) or 3 (2, 4); 5, 6 = its form with the rows staged in shared memory by
- * tensor-memory copies, where nz is a multiple of 4 and the part is large enough
- * (else as 4).  FP64: 0 = 8 voxel columns per warp at 2 blocks/SM, 1 =
+ * tensor-memory copies, where the z columns of its sinogram are whole 16 bytes
+ * (nz a multiple of 4; 8 for the iterates of BF16 storage), else as 4.  With -1 the
+ * plain operators take 5 or 4 by the same rule.  FP64: 0 = 8 voxel columns per warp at 2 blocks/SM, 1 =
  * 4 columns at 2 blocks/SM, 2-6 = 4 columns at 3 blocks/SM.  Volumes of few z
  * values have one kernel for every entry.  Every entry gives the same sums bit
  * for bit within one precision. */

@@ -5,8 +5,8 @@
 // the same sums).  What changes is where the rows come from.  A block has ROWS
 // warps = ROWS voxel rows of 4 columns; for each view it needs the bins that its
 // voxels reach: over 4 x 8 voxels floor(u) spans at most ceil(3 |cos| + 7 |sin|) + 1
-// <= 9 values, over 4 x 4 at most 6, over 4 x 2 at most 5, so a box of 10, 7 or 6 bins
-// from the block's smallest floor(u) holds every tap.  One more warp copies the
+// <= 9 values, over 4 x 2 (the other tile) at most 5, so a box of 10 or 6 bins from
+// the block's smallest floor(u) holds every tap.  One more warp copies the
 // boxes ([T z values] x [bins] of one view, cp.async.bulk.tensor; bins off the
 // detector and z beyond the column arrive as zeros) into a ring of stages, two
 // views a stage, as far ahead as the ring allows; the others read their rows from
@@ -155,7 +155,9 @@ __device__ __forceinline__ void bt_view(const SI* box, const BtEnt& e, float (&a
 }
 
 // NG groups of four z values a lane: tiles of 128 NG (nz % 4 == 0).  ROWS:
-// tiles.rows.  need, list and modes as k_backproject2.
+// tiles.rows.  need, list and modes as k_backproject2.  Two rows: 6 blocks an SM with
+// one group; with two groups of FP32 a block's 52 KB of shared memory leave 4, and the
+// bound of 6 only keeps a thread to 112 registers.
 template <typename SI, typename S, int NG, int ROWS, int MODE, typename O>
 __global__ void __launch_bounds__(32 * (ROWS + 1), ROWS == 8 ? 2 : 6)
 k_backproject_tma(const Geo<float> g, const __grid_constant__ CUtensorMap tmap, const Bufs<S, float> b,

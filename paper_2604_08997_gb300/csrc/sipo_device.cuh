@@ -90,8 +90,10 @@ template <> struct Compute<double> { using type = double; };
 // p + q * 32 * G, where p = tile start + l * G: one access of the warp to a
 // group covers 32 * G consecutive elements, so each request uses every byte of
 // its sectors (16 bytes a lane for 4-byte data, 8 for bf16, 4 for labels).
-// The host picks ZL = G or 2G only when nz is a multiple of G (and of 64 G for
-// 2G), which keeps every group access aligned and inside its z column.
+// The element-wise epilogues and the FP64 backprojector use it; launch_backproject
+// picks ZL = G only when nz is a multiple of G, and 2G when it is one of 64 G, which
+// keeps every group access aligned and inside its z column.  (ZForm below is the
+// layout of the other kernels.)
 template <typename C, int ZL>
 struct ZLayout {
   static constexpr int kVec = 16 / int(sizeof(C));
