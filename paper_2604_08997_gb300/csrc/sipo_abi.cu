@@ -202,7 +202,7 @@ struct Solver final : SolverBase {
   double* trace = nullptr;
   static constexpr int kTraceCap = 4096;
   Scal* h_st = nullptr;  // pinned host mirror
-  volatile unsigned int* h_fault = nullptr;  // fault words of the staged backprojector, mapped
+  volatile unsigned int* h_fault = nullptr;  // fault words of the staged backprojector (behind h_st, mapped)
 
   // host constants
   bool ft_is_const = false;
@@ -253,10 +253,11 @@ struct Solver final : SolverBase {
       ck(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking), "cudaStreamCreate");
       own_stream = true;
     }
-    ck(cudaHostAlloc(reinterpret_cast<void**>(&h_st), sizeof(Scal), cudaHostAllocDefault), "cudaHostAlloc");
-    unsigned int* fault = nullptr;
-    ck(cudaHostAlloc(reinterpret_cast<void**>(&fault), 2 * sizeof(unsigned int), cudaHostAllocMapped),
+    // the host mirror and, behind it, the fault words: one allocation, as each one
+    // adds a few tenths of a millisecond to the creation of a context
+    ck(cudaHostAlloc(reinterpret_cast<void**>(&h_st), sizeof(Scal) + 2 * sizeof(unsigned int), cudaHostAllocMapped),
        "cudaHostAlloc");
+    unsigned int* fault = reinterpret_cast<unsigned int*>(h_st + 1);
     fault[0] = fault[1] = 0u;
     h_fault = fault;
     unsigned int* mapped = nullptr;
@@ -270,7 +271,6 @@ struct Solver final : SolverBase {
     for (void* p : allocs) cudaFree(p);
     if (tconv) cudaFree(tconv);
     if (h_st) cudaFreeHost(h_st);
-    if (h_fault) cudaFreeHost(const_cast<unsigned int*>(h_fault));
     if (own_stream && stream) cudaStreamDestroy(stream);
   }
 

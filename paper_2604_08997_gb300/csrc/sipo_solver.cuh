@@ -299,8 +299,9 @@ __device__ __forceinline__ void dual_update(const Bufs<S, C>& b, const StepScala
 // How many neighbouring values of a ray the check step's sums add in the compute
 // type before they go to FP64: whole groups of four (all of a lane's values where
 // z columns are whole tiles of 256), else one, as narrower groups also serve
-// columns that are not whole groups of four.  The sums of a check, and with them
-// its restart and stop decisions, then do not depend on the z form.
+// columns that are not whole groups of four.  A lane of eight values then adds
+// no more of them in single precision than one of four did: restart and stop
+// decisions rest on these sums.
 template <typename C, typename Z>
 constexpr int check_fold() {
   return sizeof(C) == 8 || !Z::kRagged ? Z::ZL : (Z::G == 4 ? 4 : 1);
