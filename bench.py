@@ -60,8 +60,8 @@ def sm_max_mhz(peaks: dict) -> float:
 # the code it is null until re-captured.
 KERNEL_SOURCES = ["sipo_device.cuh", "sipo_solver.cuh", "sipo_ops.cuh", "sipo_launch.h",
                   "sipo_project.cu", "sipo_backproject.cu", "sipo_bp_tma.cuh", "sipo_pair.cuh", "sipo_wait.cuh"]
-TRAFFIC = {("csg256", "f32"): {"sources_sha256_16": "9ebeb4d949b906e3",
-                               "project": 289981696, "backproject": 218191104}}
+TRAFFIC = {("csg256", "f32"): {"sources_sha256_16": "4c24f425f5b452f5",
+                               "project": 285142784, "backproject": 216989184}}
 
 
 def _code_only(text: str) -> str:
